@@ -471,6 +471,7 @@ static SxArgs sx_args(const kin_ctx* c)
     S.nvel = c->nvel;
     S.npop = c->npop;
     S.system = c->system;
+    S.lambda = c->lambda;
     S.omega = c->omega;
     S.gamma = c->gamma;
     for (int i = 0; i < 16; ++i) S.minv[i] = c->minv[i];

@@ -3,8 +3,11 @@
 // conservation diagnostics.
 #include "kin_aux.h"
 #include "kin_device.cuh"
+#include "kin_init.cuh"
 
 #include <math.h>
+
+#include <type_traits>
 
 namespace kin {
 
@@ -150,7 +153,7 @@ __global__ void setup_kernel(SetupArgs A)
 
 // Flux in FP64 (eq. conslaw): scalar advection, Euler, or Maxwell in 3D
 // (Sec. 6.1.1: Q(W, e_a) = (-e_a x H, e_a x E), W = (E, H)).
-__host__ __device__ static void flux64(const PointArgs& A, const double* W, int a, double* Q)
+static void flux64(const PointArgs& A, const double* W, int a, double* Q)
 {
     if (A.system == kAdvection) {
         Q[0] = A.adv[a] * W[0];
@@ -178,7 +181,7 @@ __host__ __device__ static void flux64(const PointArgs& A, const double* W, int 
 }
 
 // The 2d-velocity Maxwellians of one state on the host, in FP64, with the
-// formulas of init_kernel: M[(2a + s) m + v] = W_v/(2d) +- Q^a(W)_v/(2 lambda).
+// Maxwellians of init_kernel: M[(2a + s) m + v] = W_v/(2d) +- Q^a(W)_v/(2 lambda).
 void axis_maxwellian(const PointArgs& A, const double* W, double* M)
 {
     double Q[kMaxVars];
@@ -192,23 +195,39 @@ void axis_maxwellian(const PointArgs& A, const double* W, double* M)
     }
 }
 
-// f = M(W) (Sec. 2.2 initialisation), W in FP64, f stored in T.
-template <typename T>
-__global__ void init_kernel(PointArgs A, const double* __restrict__ W, T* __restrict__ f)
+// f = M(W) (Sec. 2.2 initialisation), W in FP64, f stored in T: the 2d
+// equilibria W/(2d) +- Q^a(W)/(2 lambda), in FP64 for an FP64 state and on
+// FP32 pairs for an FP32 one (kin_init.cuh, which has the figures).  The
+// 2d m stores of a node and the m loads are all independent, one coalesced
+// access per warp each.
+template <int D, int SYS, typename T>
+__global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ InitArgs A,
+                                                        const double* __restrict__ W, T* __restrict__ f)
 {
+    constexpr int M = nvars(D, SYS);
     const long long nodes = A.nodes;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nodes;
          i += (long long)gridDim.x * blockDim.x) {
-        double w[kMaxVars], Q[kMaxVars];
-        for (int v = 0; v < A.m; ++v) w[v] = W[v * nodes + i];
-        for (int a = 0; a < A.dim; ++a) {
-            flux64(A, w, a, Q);
-            for (int v = 0; v < A.m; ++v) {
-                const double base = w[v] / (2.0 * A.dim), half = Q[v] / (2.0 * A.lambda);
-                f[((2 * a) * A.m + v) * nodes + i] = (T)(base + half);
-                f[((2 * a + 1) * A.m + v) * nodes + i] = (T)(base - half);
+        init_node<D, SYS, T>(W, nodes, i, A.fast, [&](const auto& w) {
+            using V = std::remove_cv_t<std::remove_reference_t<decltype(w[0])>>;
+            const InitK<V>& K = init_k<V>(A);
+            V Q[D][M];
+            init_flux<D, SYS, V>(K, w, Q);
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+                V base;
+                if constexpr (std::is_same<V, double>::value) base = div2d<D>(w[v]);
+                else base = w[v] * K.inv_nv;
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    // (Maxwell: Q^a has no component along E_a and H_a)
+                    const bool z = SYS == kMaxwell && (v == a || v == 3 + a);
+                    const V half = Q[a][v] * K.inv2l;
+                    init_put(f[(long long)((2 * a) * M + v) * nodes + i], z ? base : base + half);
+                    init_put(f[(long long)((2 * a + 1) * M + v) * nodes + i], z ? base : base - half);
+                }
             }
-        }
+        });
     }
 }
 
@@ -369,12 +388,44 @@ static int grid_for(long long n)
     return (int)(g < 1 ? 1 : g);
 }
 
+InitArgs init_args(long long nodes, int dim, double lambda, double gamma, const double* adv)
+{
+    InitArgs A;
+    A.nodes = nodes;
+    A.fast = init_fast_model(lambda, gamma, adv);
+    auto fill = [&](auto& K, auto make) {
+        K.gm1 = make(gamma - 1.0);
+        for (int a = 0; a < 3; ++a) K.adv[a] = make(adv[a]);
+        K.inv_nv = make(1.0 / (2.0 * dim));
+        K.inv2l = make(1.0 / (2.0 * lambda));
+    };
+    fill(A.kd, [](double x) { return x; });
+    fill(A.kf, [](double x) { return f2_make(x); });
+    return A;
+}
+
+template <int D, int SYS>
+static cudaError_t init_dispatch(const InitArgs& A, const double* W, void* f, int prec, int g, cudaStream_t st)
+{
+    if (prec == 1) init_kernel<D, SYS, float><<<g, kThreads, 0, st>>>(A, W, (float*)f);
+    else init_kernel<D, SYS, double><<<g, kThreads, 0, st>>>(A, W, (double*)f);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_init(const PointArgs& a, const double* W, void* f, int prec, cudaStream_t st)
 {
-    int g = grid_for(a.nodes);
-    if (prec == 1) init_kernel<float><<<g, kThreads, 0, st>>>(a, W, (float*)f);
-    else init_kernel<double><<<g, kThreads, 0, st>>>(a, W, (double*)f);
-    return cudaGetLastError();
+    const int g = grid_for(a.nodes);
+    const InitArgs A = init_args(a.nodes, a.dim, a.lambda, a.gamma, a.adv);
+    switch (a.dim * 4 + a.system) {
+    case 4: return init_dispatch<1, kAdvection>(A, W, f, prec, g, st);
+    case 5: return init_dispatch<1, kEuler>(A, W, f, prec, g, st);
+    case 8: return init_dispatch<2, kAdvection>(A, W, f, prec, g, st);
+    case 9: return init_dispatch<2, kEuler>(A, W, f, prec, g, st);
+    case 12: return init_dispatch<3, kAdvection>(A, W, f, prec, g, st);
+    case 13: return init_dispatch<3, kEuler>(A, W, f, prec, g, st);
+    case 14: return init_dispatch<3, kMaxwell>(A, W, f, prec, g, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_moments(const PointArgs& a, const void* f, double* W, int prec, cudaStream_t st)

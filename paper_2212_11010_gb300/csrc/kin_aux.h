@@ -69,7 +69,7 @@ struct SxArgs {
     int dim, degree, nn, m, nvel, npop, system;
     int from_f;                   // iterate 1: interface inflow is f^n of the upwind cell
     int final_iter;
-    double omega, gamma;
+    double lambda, omega, gamma;
     double adv[3];
     double minv[16];
 };

@@ -20,10 +20,13 @@
 //                precomputed in FP64).
 #include "kin_aux.h"
 #include "kin_device.cuh"
+#include "kin_init.cuh"
 #include "kin_tma.cuh"
 
 #include <math.h>
 #include <string.h>
+
+#include <type_traits>
 
 namespace kin {
 
@@ -830,36 +833,42 @@ __global__ void sx_relax_kernel(SxArgs S)
     }
 }
 
-// f = M(W) for the d + 1 sets (initialisation), FP64 in.
+// f = M(W) for the d + 1 sets (initialisation), FP64 in; the arithmetic is
+// that of kin_init.cuh.  md / mf: the inverse moment matrix in FP64 / as pairs.
+template <int NV>
+struct SxInit {
+    InitArgs A;
+    double md[NV * NV];
+    F2 mf[NV * NV];
+};
+
 template <int D, int SYS, typename T>
-__global__ void sx_init_kernel(SxArgs S, const double* __restrict__ Wd)
+__global__ void __launch_bounds__(256) sx_init_kernel(const __grid_constant__ SxInit<D + 1> S,
+                                                      const double* __restrict__ Wd, T* __restrict__ f)
 {
     constexpr int M = nvars(D, SYS);
     constexpr int NV = D + 1;
-    T* f = static_cast<T*>(S.f);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.nodes;
+    const long long nodes = S.A.nodes;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nodes;
          i += (long long)gridDim.x * blockDim.x) {
-        double W[M], Q[D][M];
-        for (int v = 0; v < M; ++v) W[v] = Wd[(long long)v * S.nodes + i];
-        if (SYS == kAdvection) {
-            for (int a = 0; a < D; ++a) Q[a][0] = S.adv[a] * W[0];
-        } else {
-            double ke = 0.0;
-            for (int b = 0; b < D; ++b) ke += W[1 + b] * W[1 + b];
-            const double pr = (S.gamma - 1.0) * (W[1 + D] - 0.5 * ke / W[0]);
-            for (int a = 0; a < D; ++a) {
-                const double ua = W[1 + a] / W[0];
-                Q[a][0] = W[1 + a];
-                for (int b = 0; b < D; ++b) Q[a][1 + b] = W[1 + b] * ua + (b == a ? pr : 0.0);
-                Q[a][1 + D] = (W[1 + D] + pr) * ua;
-            }
-        }
-        for (int kk = 0; kk < NV; ++kk)
-            for (int v = 0; v < M; ++v) {
-                double mk = S.minv[kk * NV] * W[v];
-                for (int a = 0; a < D; ++a) mk += S.minv[kk * NV + 1 + a] * Q[a][v];
-                f[(long long)(kk * M + v) * S.nodes + i] = (T)mk;
-            }
+        init_node<D, SYS, T>(Wd, nodes, i, S.A.fast, [&](const auto& W) {
+            using V = std::remove_cv_t<std::remove_reference_t<decltype(W[0])>>;
+            V Q[D][M];
+            init_flux<D, SYS, V>(init_k<V>(S.A), W, Q);
+#pragma unroll
+            for (int kk = 0; kk < NV; ++kk)
+#pragma unroll
+                for (int v = 0; v < M; ++v) {
+                    auto mi = [&](int j) {
+                        if constexpr (std::is_same<V, double>::value) return S.md[kk * NV + j];
+                        else return S.mf[kk * NV + j];
+                    };
+                    V mk = mi(0) * W[v];
+#pragma unroll
+                    for (int a = 0; a < D; ++a) mk = mk + mi(1 + a) * Q[a][v];
+                    init_put(f[(long long)(kk * M + v) * nodes + i], mk);
+                }
+        });
     }
 }
 
@@ -1044,13 +1053,25 @@ cudaError_t sx_launch_trace0(const SxArgs& a, int prec, cudaStream_t st)
     return cudaGetLastError();
 }
 
+template <int D, int SYS, typename T>
+static void init_go(const SxArgs& a, const double* W, int g, cudaStream_t st)
+{
+    SxInit<D + 1> S;
+    S.A = init_args(a.nodes, a.dim, a.lambda, a.gamma, a.adv);
+    for (int i = 0; i < (D + 1) * (D + 1); ++i) {
+        S.md[i] = a.minv[i];
+        S.mf[i] = f2_make(a.minv[i]);
+    }
+    sx_init_kernel<D, SYS, T><<<g, 256, 0, st>>>(S, W, static_cast<T*>(a.f));
+}
+
 template <typename T>
 static cudaError_t relax_dispatch(const SxArgs& a, cudaStream_t st, bool init, const double* W)
 {
     const int g = sx_grid(a.nodes);
 #define KIN_SX(DD, SY)                                                                     \
     if (a.dim == DD && a.system == SY) {                                                   \
-        if (init) sx_init_kernel<DD, SY, T><<<g, 256, 0, st>>>(a, W);                      \
+        if (init) init_go<DD, SY, T>(a, W, g, st);                      \
         else sx_relax_kernel<DD, SY, T><<<g, 256, 0, st>>>(a);                             \
         return cudaGetLastError();                                                         \
     }

@@ -26,6 +26,7 @@
 // inside (eq. ibvp); iterate 0 is f^n.
 #include "kin_aux.h"
 #include "kin_device.cuh"
+#include "kin_init.cuh"
 
 #include <algorithm>
 #include <type_traits>
@@ -378,21 +379,47 @@ __global__ void __launch_bounds__(256) tet_relax_kernel(TetArgs A, const T* __re
     }
 }
 
-// f = M(W) from the FP64 macroscopic state (Sec. 2.2 initialisation).
+// f = M(W) from the FP64 macroscopic state (Sec. 2.2 initialisation), the
+// equilibria of tet_equilibria in the arithmetic of kin_init.cuh.
 template <int SYS, int VS, typename T>
-__global__ void tet_init_kernel(TetArgs A, const double* __restrict__ W0)
+__global__ void __launch_bounds__(256) tet_init_kernel(const __grid_constant__ InitArgs A,
+                                                       const double* __restrict__ W0, T* __restrict__ f)
 {
-    constexpr int m = nvars(3, SYS), NPOP = (VS == 1 ? 4 : 6) * m;
-    T* f = static_cast<T*>(A.f);
+    constexpr int m = nvars(3, SYS);
     const long long nodes = A.nodes;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nodes;
          i += (long long)gridDim.x * blockDim.x) {
-        double W[m], M[NPOP];
+        init_node<3, SYS, T>(W0, nodes, i, A.fast, [&](const auto& W) {
+            using V = std::remove_cv_t<std::remove_reference_t<decltype(W[0])>>;
+            const InitK<V>& K = init_k<V>(A);
+            V Q[3][m];
+            init_flux<3, SYS, V>(K, W, Q);
 #pragma unroll
-        for (int v = 0; v < m; ++v) W[v] = W0[v * nodes + i];
-        tet_equilibria<SYS, VS>(A, W, M);
+            for (int v = 0; v < m; ++v) {
+                if constexpr (VS == 1) {
+                    // 1 / (4 lambda) and 1/4: halves of the constants of the axis set with d = 2
+                    const V half = init_const<V>(0.5), base = W[v] * init_const<V>(0.25);
+                    const V il = K.inv2l * half;
+                    const V qx = Q[0][v] * il, qy = Q[1][v] * il, qz = Q[2][v] * il;
+                    const V a = base + qx, b = base - qx, s = qy + qz, d = qy - qz;
+                    // signs (+,+,+), (+,-,-), (-,+,-), (-,-,+)
+                    init_put(f[(long long)(0 * m + v) * nodes + i], a + s);
+                    init_put(f[(long long)(1 * m + v) * nodes + i], a - s);
+                    init_put(f[(long long)(2 * m + v) * nodes + i], b + d);
+                    init_put(f[(long long)(3 * m + v) * nodes + i], b - d);
+                } else {
+                    V base;
+                    if constexpr (std::is_same<V, double>::value) base = div2d<3>(W[v]);
+                    else base = W[v] * K.inv_nv;
 #pragma unroll
-        for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = (T)M[p];
+                    for (int a = 0; a < 3; ++a) {
+                        const V q = Q[a][v] * K.inv2l;
+                        init_put(f[(long long)((2 * a) * m + v) * nodes + i], base + q);
+                        init_put(f[(long long)((2 * a + 1) * m + v) * nodes + i], base - q);
+                    }
+                }
+            }
+        });
     }
 }
 
@@ -429,7 +456,8 @@ template <int S, int V, typename T>
 struct InitLaunch {
     static void launch(const TetArgs& a, unsigned grid, cudaStream_t st, const double* W)
     {
-        tet_init_kernel<S, V, T><<<grid, 256, 0, st>>>(a, W);
+        const InitArgs A = init_args(a.nodes, 3, a.lambda, a.gamma, a.adv);
+        tet_init_kernel<S, V, T><<<grid, 256, 0, st>>>(A, W, static_cast<T*>(a.f));
     }
 };
 
