@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstdarg>
 #include <cstdio>
@@ -15,6 +16,7 @@
 #include <climits>
 #include <cstring>
 #include <string>
+#include <thread>
 #include <vector>
 
 using namespace kin;
@@ -78,6 +80,9 @@ struct kin_ctx {
     int* tlstart = nullptr;           // [velocity][nsub + 1]
     int* tbounds = nullptr;           // level boundaries
     int* tfref = nullptr;             // [velocity][position][4] packed inflow face references
+    int* thstart = nullptr;           // ring sweep: interface cells of every chunk
+    int* thcell = nullptr;
+    TetPlan tplan = {};
     void* titer[2] = {nullptr, nullptr};   // subdomain iterates
     std::vector<double> tvol;         // host: cell volumes, for the mass diagnostic
     bool have_state = false;
@@ -525,6 +530,9 @@ static TetArgs tet_args(const kin_ctx* c)
     a.lstart = c->tlstart;
     a.bounds = c->tbounds;
     a.fref = c->tfref;
+    a.hstart = c->thstart;
+    a.hcell = c->thcell;
+    a.plan = c->tplan;
     a.f = c->f;
     a.lambda = c->lambda;
     a.gamma = c->gamma;
@@ -537,18 +545,48 @@ static TetArgs tet_args(const kin_ctx* c)
 }
 
 // One step S(dt) on a tetrahedral mesh: K sweeps (iterate p in titer[p & 1],
-// iterate 0 = f^n), then the Crank-Nicolson extrapolation with the
-// relaxation.
+// iterate 0 = f^n), then the relaxation.  With the ring sweep the last of
+// several iterates writes f^{n+1} in place (no other block reads f then: the
+// interface values come from titer) and the others only what the neighbours
+// read; else the relaxation extrapolates from f*.
 static kin_status tet_step(kin_ctx* c)
 {
     const TetArgs a = tet_args(c);
     const int prec = c->precision == KIN_FP32;
+    const int in_place = c->tplan.chunk > 0 && c->iters > 1;
     for (int p = 1; p <= c->iters; ++p) {
         const void* prev = p == 1 ? c->f : c->titer[(p - 1) & 1];
-        KIN_CUDA(c, tet_launch_sweep(a, prev, c->titer[p & 1], prec, c->stream));
+        KIN_CUDA(c, tet_launch_sweep(a, prev, c->titer[p & 1], in_place && p == c->iters, !in_place, prec, c->stream));
     }
-    KIN_CUDA(c, tet_launch_relax(a, c->titer[c->iters & 1], prec, c->stream));
+    KIN_CUDA(c, tet_launch_relax(a, in_place ? nullptr : c->titer[c->iters & 1], prec, c->stream));
     return KIN_OK;
+}
+
+// fn(0) .. fn(nvel - 1), one host thread each (the caller's for the last, and
+// for those that could not be started); false when one threw (out of memory).
+template <typename F>
+static bool each_velocity(int nvel, const F& fn)
+{
+    std::atomic<bool> ok{true};
+    auto body = [&](int k) {
+        try {
+            fn(k);
+        } catch (...) {
+            ok = false;
+        }
+    };
+    std::thread th[6];
+    for (int k = 0; k < nvel; ++k) {
+        try {
+            if (k + 1 < nvel && k < 6) th[k] = std::thread(body, k);
+            else body(k);
+        } catch (...) {
+            body(k);
+        }
+    }
+    for (auto& t : th)
+        if (t.joinable()) t.join();
+    return ok;
 }
 
 extern "C" {
@@ -998,70 +1036,179 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
             ftype[(size_t)k * n + cc] = t;
         }
     }
-    // breadth-first levels of every subdomain's oriented graph, per velocity
-    std::vector<int> order((size_t)c->nvel * n), lstart((size_t)c->nvel * (nsub + 1)), bounds;
+    // breadth-first levels of every subdomain's oriented graph.  The velocities
+    // are independent of one another here and in the face references below: one
+    // host thread each.
+    std::vector<int> order((size_t)c->nvel * n), rank((size_t)c->nvel * n), lstart, bounds;
+    auto inflow = [&](int k, int cc, int a) { return ((ftype[(size_t)k * n + cc] >> (2 * a)) & 3) == 1; };
+    struct Levels {
+        std::vector<int> lstart, bounds;                 // of one velocity; positions are the velocity's own
+        int cycle = -1;                                  // a subdomain with a cycle
+        int ring = 1, width = 1, levels = 1, cells = 1;  // what the ring sweep has to hold
+    };
+    std::vector<Levels> lv(c->nvel);
+    std::vector<int> bysub(n), sstart(nsub + 1, 0);
+    for (int cc = 0; cc < n; ++cc) sstart[mesh->sub[cc] + 1]++;
+    for (int q = 0; q < nsub; ++q) sstart[q + 1] += sstart[q];
     {
-        std::vector<int> bysub(n), sstart(nsub + 1, 0);
-        for (int cc = 0; cc < n; ++cc) sstart[mesh->sub[cc] + 1]++;
-        for (int q = 0; q < nsub; ++q) sstart[q + 1] += sstart[q];
         std::vector<int> fill(sstart.begin(), sstart.end() - 1);
         for (int cc = 0; cc < n; ++cc) bysub[fill[mesh->sub[cc]]++] = cc;
-        std::vector<int> indeg(n), lev(n);
-        for (int k = 0; k < c->nvel; ++k) {
-            int* ord = order.data() + (size_t)k * n;
-            for (int cc = 0; cc < n; ++cc) {
-                indeg[cc] = 0;
-                lev[cc] = 0;
-                for (int a = 0; a < 4; ++a)
-                    if (((ftype[(size_t)k * n + cc] >> (2 * a)) & 3) == 1 && !((iface[cc] >> a) & 1)) indeg[cc]++;
-            }
-            int pos = 0;
-            for (int q = 0; q < nsub; ++q) {
-                lstart[(size_t)k * (nsub + 1) + q] = (int)bounds.size();
-                const int head0 = pos;
-                for (int i = sstart[q]; i < sstart[q + 1]; ++i)
-                    if (indeg[bysub[i]] == 0) ord[pos++] = bysub[i];
-                int head = head0;
-                while (head < pos) {
-                    const int cc = ord[head++];
-                    for (int a = 0; a < 4; ++a) {
-                        if (((ftype[(size_t)k * n + cc] >> (2 * a)) & 3) != 2 || ((iface[cc] >> a) & 1)) continue;
-                        const int R = (int)mesh->nbr[(size_t)cc * 4 + a];
-                        lev[R] = std::max(lev[R], lev[cc] + 1);
-                        if (--indeg[R] == 0) ord[pos++] = R;
-                    }
-                }
-                if (pos - head0 != sstart[q + 1] - sstart[q]) {
-                    delete c;
-                    return fail(nullptr, KIN_EINVAL, "subdomain %d: the oriented cell graph of velocity %d has a cycle "
-                                "(a subdomain wrapping the periodic box needs its wrap faces marked)", q, k);
-                }
-                // the breadth-first order lists the cells level by level
-                std::stable_sort(ord + head0, ord + pos, [&](int x, int y) { return lev[x] < lev[y]; });
-                for (int i = head0; i < pos; ++i)
-                    if (i == head0 || lev[ord[i]] != lev[ord[i - 1]]) bounds.push_back(i);
-            }
-            lstart[(size_t)k * (nsub + 1) + nsub] = (int)bounds.size();
-            bounds.push_back(pos);
-        }
     }
-    // inflow faces per (velocity, position in its order), one word each:
-    // the neighbour cell R << 7, the neighbour's local index (2 bits) of
-    // each of the face's three vertices at bits 5, 3 and 1, and bit 0 set
-    // when the face is a subdomain interface; -1 on the faces that are not
-    // inflow faces (R < 2^24 by the cell-count check above)
-    std::vector<int> fref((size_t)c->nvel * n * 4, -1);
-    for (int k = 0; k < c->nvel; ++k)
-        for (int q = 0; q < n; ++q) {
-            const int cc = order[(size_t)k * n + q];
-            for (int a = 0; a < 4; ++a) {
-                if (((ftype[(size_t)k * n + cc] >> (2 * a)) & 3) != 1) continue;
-                const int R = fnodes[(size_t)cc * 12 + a * 3] / 4;
-                int wd = (R << 7) | ((iface[cc] >> a) & 1);
-                for (int jj = 0; jj < 3; ++jj) wd |= (fnodes[(size_t)cc * 12 + a * 3 + jj] & 3) << (5 - 2 * jj);
-                fref[((size_t)k * n + q) * 4 + a] = wd;
+    bool ran = each_velocity(c->nvel, [&](int k) {
+        Levels& V = lv[k];
+        const unsigned char* ft = ftype.data() + (size_t)k * n;
+        int *ord = order.data() + (size_t)k * n, *rk = rank.data() + (size_t)k * n;
+        std::vector<int> indeg(n, 0), lev(n, 0);
+        for (int cc = 0; cc < n; ++cc)
+            for (int a = 0; a < 4; ++a)
+                if (inflow(k, cc, a) && !((iface[cc] >> a) & 1)) indeg[cc]++;
+        std::vector<std::vector<int>> bucket;            // a level's cells by inflow faces
+        int pos = 0;
+        for (int q = 0; q < nsub; ++q) {
+            V.lstart.push_back((int)V.bounds.size());
+            const int head0 = pos;
+            for (int i = sstart[q]; i < sstart[q + 1]; ++i)
+                if (indeg[bysub[i]] == 0) ord[pos++] = bysub[i];
+            int head = head0;
+            while (head < pos) {
+                const int cc = ord[head++];
+                for (int a = 0; a < 4; ++a) {
+                    if (((ft[cc] >> (2 * a)) & 3) != 2 || ((iface[cc] >> a) & 1)) continue;
+                    const int R = (int)mesh->nbr[(size_t)cc * 4 + a];
+                    lev[R] = std::max(lev[R], lev[cc] + 1);
+                    if (--indeg[R] == 0) ord[pos++] = R;
+                }
+            }
+            if (pos - head0 != sstart[q + 1] - sstart[q]) {
+                V.cycle = q;
+                return;
+            }
+            // the order lists the cells level by level; inside a level, cells
+            // with the same inflow faces stand together, so that the cells of a
+            // warp take the same branches
+            for (int i = head0; i < pos; ++i) {
+                const int cc = ord[i];
+                int mask = 0;
+                for (int a = 0; a < 4; ++a) mask |= inflow(k, cc, a) << a;
+                const size_t key = (size_t)lev[cc] * 16 + mask;
+                if (bucket.size() <= key) bucket.resize((size_t)(lev[cc] + 1) * 16);
+                bucket[key].push_back(cc);
+            }
+            int p = head0;
+            for (size_t key = 0; key < bucket.size(); ++key) {
+                if (key % 16 == 0 && p < pos) V.bounds.push_back(p);
+                for (int cc : bucket[key]) {
+                    rk[cc] = p;
+                    ord[p++] = cc;
+                }
+                bucket[key].clear();
+            }
+            // The ring sweep keeps the last 'ring' cells of a subdomain's
+            // order: a cell's slot may be reused once no cell of the writing
+            // level or a later one reads it, i.e. level end - earliest
+            // position read from there on.
+            const int l0 = V.lstart.back(), l1 = (int)V.bounds.size();
+            int minref = n, end = pos;
+            for (int l = l1 - 1; l >= l0; --l) {
+                for (int i = V.bounds[l]; i < end; ++i)
+                    for (int a = 0; a < 4; ++a)
+                        if (inflow(k, ord[i], a) && !((iface[ord[i]] >> a) & 1))
+                            minref = std::min(minref, rk[mesh->nbr[(size_t)ord[i] * 4 + a]]);
+                V.width = std::max(V.width, end - V.bounds[l]);
+                V.ring = std::max(V.ring, end - std::min(minref, V.bounds[l]));
+                end = V.bounds[l];
+            }
+            V.levels = std::max(V.levels, l1 - l0);
+            V.cells = std::max(V.cells, pos - head0);
+        }
+        V.lstart.push_back((int)V.bounds.size());
+        V.bounds.push_back(pos);
+    });
+    Levels most;
+    for (int k = 0; ran && k < c->nvel; ++k) {
+        if (lv[k].cycle >= 0) {
+            const int q = lv[k].cycle;
+            delete c;
+            return fail(nullptr, KIN_EINVAL, "subdomain %d: the oriented cell graph of velocity %d has a cycle "
+                        "(a subdomain wrapping the periodic box needs its wrap faces marked)", q, k);
+        }
+        most.ring = std::max(most.ring, lv[k].ring);
+        most.width = std::max(most.width, lv[k].width);
+        most.levels = std::max(most.levels, lv[k].levels);
+        most.cells = std::max(most.cells, lv[k].cells);
+    }
+    if (!tet_make_plan(most.ring, most.width, most.levels, most.cells, nsub * c->nvel, c->m,
+                       c->precision == KIN_FP32, &c->tplan))
+        c->tplan = TetPlan{};
+    // inflow faces per (velocity, position in its order), one word each: the
+    // source << 7, the neighbour's local index (2 bits) of each of the face's
+    // three vertices at bits 5, 3 and 1, and bit 0 set when the face is a
+    // subdomain interface; -1 on the faces that are not inflow faces.  The
+    // source is the neighbour cell (< 2^24 by the cell-count check above); for
+    // the ring sweep, whose levels are cut into chunks here, the neighbour's
+    // ring slot or its place among the chunk's interface cells.
+    std::vector<int> fref((size_t)c->nvel * n * 4, -1), hstart, hcell;
+    struct Chunks {
+        std::vector<int> start, bounds, hstart, hcell;
+    };
+    std::vector<Chunks> cks(c->nvel);
+    ran = ran && each_velocity(c->nvel, [&](int k) {
+        const Levels& V = lv[k];
+        Chunks& K = cks[k];
+        int *ord = order.data() + (size_t)k * n, *fr = fref.data() + (size_t)k * n * 4;
+        const int *rk = rank.data() + (size_t)k * n, C = c->tplan.chunk, R = std::max(1, c->tplan.ring);
+        for (int s = 0; s < nsub; ++s) {
+            const int start = V.bounds[V.lstart[s]];
+            K.start.push_back((int)K.bounds.size());
+            for (int l = V.lstart[s]; l < V.lstart[s + 1]; ++l) {
+                int cells = C;                           // cells of the open chunk (C: none is open)
+                for (int q = V.bounds[l]; q < V.bounds[l + 1]; ++q) {
+                    const int cc = ord[q];
+                    int nh = 0, out = 0;
+                    for (int a = 0; a < 4; ++a) nh += inflow(k, cc, a) && ((iface[cc] >> a) & 1);
+                    if (C == 0 ? q == V.bounds[l] : cells == C || (int)K.hcell.size() - K.hstart.back() + nh > C) {
+                        K.bounds.push_back(q);
+                        K.hstart.push_back((int)K.hcell.size());
+                        cells = 0;
+                    }
+                    ++cells;
+                    for (int a = 0; a < 4; ++a) {
+                        const int R0 = (int)mesh->nbr[(size_t)cc * 4 + a];
+                        const bool itf = (iface[cc] >> a) & 1;
+                        if (!inflow(k, cc, a)) {
+                            if (itf) out = kTetOutFace;
+                            continue;
+                        }
+                        int src = R0;
+                        if (C > 0 && itf) {
+                            src = (int)K.hcell.size() - K.hstart.back();
+                            K.hcell.push_back(R0);
+                        } else if (C > 0) {
+                            src = (rk[R0] - start) % R;
+                        }
+                        int wd = (src << 7) | (int)itf;
+                        for (int jj = 0; jj < 3; ++jj)
+                            wd |= (fnodes[(size_t)cc * 12 + a * 3 + jj] & 3) << (5 - 2 * jj);
+                        fr[(size_t)q * 4 + a] = wd;
+                    }
+                    if (C > 0) ord[q] |= out;
+                }
             }
         }
+        K.start.push_back((int)K.bounds.size());
+        K.bounds.push_back(n);
+        K.hstart.push_back((int)K.hcell.size());
+    });
+    if (!ran) {
+        delete c;
+        return fail(nullptr, KIN_ENOMEM, "host allocation failed");
+    }
+    for (const Chunks& K : cks) {
+        for (int l : K.start) lstart.push_back(l + (int)bounds.size());
+        for (int h : K.hstart) hstart.push_back(h + (int)hcell.size());
+        bounds.insert(bounds.end(), K.bounds.begin(), K.bounds.end());
+        hcell.insert(hcell.end(), K.hcell.begin(), K.hcell.end());
+    }
 
     kin_status st;
     void* p;
@@ -1083,6 +1230,10 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
     ALLOC(c->tlstart, sizeof(int) * lstart.size());
     ALLOC(c->tbounds, sizeof(int) * bounds.size());
     ALLOC(c->tfref, sizeof(int) * fref.size());
+    if (c->tplan.chunk > 0) {
+        ALLOC(c->thstart, sizeof(int) * hstart.size());
+        ALLOC(c->thcell, sizeof(int) * hcell.size());
+    }
     ALLOC(c->Wbuf, sizeof(double) * c->m * c->nodes);
     ALLOC(c->errword, sizeof(int) * 4);
     // FP64 setup scratch: vertex coordinates, face types, FP64 records
@@ -1095,9 +1246,6 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
     int* rank_d = nullptr;
     ALLOC(rank_d, sizeof(int) * (size_t)c->nvel * n);
 #undef ALLOC
-    std::vector<int> rank((size_t)c->nvel * n);
-    for (int k = 0; k < c->nvel; ++k)
-        for (int q = 0; q < n; ++q) rank[(size_t)k * n + order[(size_t)k * n + q]] = q;
     cudaError_t e = cudaMemcpyAsync(c->torder, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->tlstart, lstart.data(), sizeof(int) * lstart.size(), cudaMemcpyHostToDevice, c->stream);
@@ -1105,6 +1253,12 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
         e = cudaMemcpyAsync(c->tbounds, bounds.data(), sizeof(int) * bounds.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->tfref, fref.data(), sizeof(int) * fref.size(), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && c->tplan.chunk > 0) {
+        e = cudaMemcpyAsync(c->thstart, hstart.data(), sizeof(int) * hstart.size(), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->thcell, hcell.data(), sizeof(int) * hcell.size(), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = tet_configure(c->tplan, c->precision == KIN_FP32);
+    }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(xyz_d, mesh->xyz, sizeof(double) * 12 * (size_t)n, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ft_d, ftype.data(), ftype.size(), cudaMemcpyHostToDevice, c->stream);
@@ -1145,8 +1299,9 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
         c->bytes_held -= b.second;
         c->blocks.pop_back();
     }
-    c->grid = (int)(c->nsub * c->nvel);
-    c->threads = kTetSweepThreads;
+    c->grid = (int)(c->nsub * c->nvel) * std::max(1, c->tplan.groups);
+    c->threads = c->tplan.chunk > 0 ? c->tplan.threads : kTetSweepThreads;
+    c->smem = (int)c->tplan.smem;
     *out = c;
     return KIN_OK;
 }

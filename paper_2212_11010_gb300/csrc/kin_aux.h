@@ -91,8 +91,10 @@ cudaError_t sx_launch_relax(const SxArgs& a, int prec, cudaStream_t st);
 cudaError_t sx_launch_init(const SxArgs& a, const double* W, int prec, cudaStream_t st);
 
 // ---- tetrahedral meshes (kin_tet.cu) ----
-constexpr int kTetRec = 21;       // coefficient slots per (velocity, cell): A^{-1}, |L|/20, four face factors
+constexpr int kTetRec = 20;       // coefficients per (velocity, cell): A^{-1} |L|/20, four face factors
 constexpr int kTetSweepThreads = 640;
+constexpr int kTetRingThreads = 768;  // bound on the ring sweep's block (and so on its registers)
+constexpr int kTetAhead = 2;      // ring sweep: chunks whose data are in flight while one is solved
 
 struct TetSetupArgs {
     int ncells, nvel;
@@ -105,23 +107,49 @@ struct TetSetupArgs {
     float* c32;                   // FP32 copy (NULL for FP64)
 };
 
+// How a sweep is run.  chunk > 0: the ring sweep -- a block takes mv variables
+// of one (subdomain, velocity) and keeps the iterate's last 'ring' cells in
+// shared memory; a level is cut into chunks of at most 'chunk' cells and as
+// many interface faces.  chunk = 0: the iterate lives in global memory.
+struct TetPlan {
+    int chunk, mv, vpt, groups, ring, desc, threads;   // desc: 16-byte words of the chunk table
+    size_t smem;
+};
+
 struct TetArgs {
     int ncells, nvel, m, npop, nsub, system, velset;
     long long nodes;              // 4 ncells
     const void* coef;             // T records [velocity][position in order][kTetRec]
-    const int* order;             // [velocity][ncells]: cells by subdomain, then breadth-first
-    const int* lstart;            // [velocity][nsub + 1]: first level index of each subdomain in bounds
-    const int* bounds;            // level l of the order holds positions [bounds[l], bounds[l + 1])
-    const int* fref;              // [velocity][position][face a]: neighbour cell << 7 | its local index of
-                                  // the face's vertices (bits 5, 3, 1) | 1 at an interface; -1 if not inflow
+    const int* order;             // [velocity][ncells]: cells by subdomain, then breadth-first; the ring sweep's
+                                  // entries carry kTetOutFace where a neighbour reads the cell across an interface
+    const int* lstart;            // [velocity][nsub + 1]: first level (chunk) index of each subdomain in bounds
+    const int* bounds;            // level (chunk) l of the order holds positions [bounds[l], bounds[l + 1])
+    const int* fref;              // [velocity][position][face a]: source << 7 | its local index of the face's
+                                  // vertices (bits 5, 3, 1) | 1 at an interface; -1 if not inflow.  Source: the
+                                  // neighbour cell, or for the ring sweep its ring slot (its place in the chunk's
+                                  // list of interface cells at an interface)
+    const int* hstart;            // ring sweep: chunk l's interface cells are hcell[hstart[l] .. hstart[l + 1])
+    const int* hcell;
+    TetPlan plan;
     void* f;                      // T [pop][cell][4]
     double lambda, gamma, omega, mu;
     double adv[3];
     int sgn[4][3];                // D3Q4 velocity signs
 };
+constexpr int kTetOutFace = 1 << 30;
+
+// The ring sweep's plan for a mesh whose iterate needs 'ring' cells resident
+// and whose subdomains have at most 'cells' cells in 'levels' levels of at
+// most 'width' cells; false when no shape fits shared memory.
+bool tet_make_plan(int ring, int width, int levels, int cells, int blocks, int m, int prec, TetPlan* plan);
+cudaError_t tet_configure(const TetPlan& plan, int prec);
 
 cudaError_t tet_launch_setup(const TetSetupArgs& a, cudaStream_t st);
-cudaError_t tet_launch_sweep(const TetArgs& a, const void* prev, void* cur, int prec, cudaStream_t st);
+// One iterate.  final: f^{n+1} = 2 f* - f^n replaces f (ring sweep, K > 1);
+// else the iterate goes to cur -- whole, or only what the neighbours read.
+cudaError_t tet_launch_sweep(const TetArgs& a, const void* prev, void* cur, int final, int whole, int prec,
+                             cudaStream_t st);
+// star: f* still to be extrapolated, or NULL when f holds f^{n+1} already
 cudaError_t tet_launch_relax(const TetArgs& a, const void* star, int prec, cudaStream_t st);
 cudaError_t tet_launch_init(const TetArgs& a, const double* W, int prec, cudaStream_t st);
 

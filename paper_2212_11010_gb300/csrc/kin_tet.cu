@@ -17,16 +17,16 @@
 // Downwind order (Sec. 3.2): for each velocity the host orients the faces,
 // and inside every subdomain sorts the cells breadth-first into levels
 // (cells of one level have no upwind neighbour in the same level).  A step
-// is K launches of the sweep kernel -- one block per (subdomain, velocity),
-// walking the levels with a barrier between them, every thread one (cell,
-// variable) pair of the level -- and one pointwise launch for the
-// Crank-Nicolson extrapolation and the relaxation.  Iteration p reads the
+// is K launches of a sweep kernel -- blocks walk the levels of a (subdomain,
+// velocity) with a barrier between them, every thread one (cell, variable)
+// pair of the level -- and one pointwise launch for the relaxation.  Iteration p reads the
 // neighbour's iterate p-1 across a subdomain interface (a face to another
 // subdomain, or across the periodic boundary) and the current iterate
 // inside (eq. ibvp); iterate 0 is f^n.
 #include "kin_aux.h"
 #include "kin_device.cuh"
 #include "kin_init.cuh"
+#include "kin_tma.cuh"
 
 #include <algorithm>
 #include <type_traits>
@@ -35,8 +35,10 @@ namespace kin {
 
 // ---------------------------------------------------------------------------
 // FP64 setup: per (velocity, cell) the record
-//   [0, 16)  A^{-1} (row-major)      [16]  |L| / 20
-//   [17, 21) tau |V.N_a| |F_a| / 12 on inflow faces a, else 0
+//   [0, 16)  B = |L|/20 A^{-1} (row-major)
+//   [16, 20) tau |V.N_a| |F_a| / 12 / (|L|/20) on inflow faces a, else 0
+// (the cell's mass factor |L|/20 is moved into both, which makes a record
+// five 16-byte words in FP32)
 // ---------------------------------------------------------------------------
 
 __global__ void tet_setup_kernel(TetSetupArgs A)
@@ -122,9 +124,8 @@ __global__ void tet_setup_kernel(TetSetupArgs A)
     const size_t pos = (size_t)A.rank[(size_t)k * A.ncells + c];
     double* rec = A.c64 + ((size_t)k * A.ncells + pos) * kTetRec;
     for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) rec[i * 4 + j] = M[i][4 + j];
-    rec[16] = vol / 20.0;
-    for (int a = 0; a < 4; ++a) rec[17 + a] = cin[a];
+        for (int j = 0; j < 4; ++j) rec[i * 4 + j] = M[i][4 + j] * (vol / 20.0);
+    for (int a = 0; a < 4; ++a) rec[16 + a] = cin[a] / (vol / 20.0);
     if (A.c32) {
         float* r32 = A.c32 + ((size_t)k * A.ncells + pos) * kTetRec;
         for (int q = 0; q < kTetRec; ++q) r32[q] = (float)rec[q];
@@ -132,7 +133,8 @@ __global__ void tet_setup_kernel(TetSetupArgs A)
 }
 
 // ---------------------------------------------------------------------------
-// sweep: one block per (subdomain, velocity), levels in order
+// sweep with the iterate in global memory: one block per (subdomain,
+// velocity), levels in order.  For subdomains too wide for the ring sweep.
 // ---------------------------------------------------------------------------
 
 // The four node values of a cell as one vector access (FP32: 16 bytes; the
@@ -205,10 +207,9 @@ __global__ void __launch_bounds__(kTetSweepThreads, 2) tet_sweep_kernel(TetArgs 
             du[i] = u[i] - r;
             sum += du[i];
         }
-        const T m20 = rec[16];
         T rhs[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) rhs[i] = m20 * (sum + du[i]);
+        for (int i = 0; i < 4; ++i) rhs[i] = sum + du[i];
         const int fw[4] = {nr.x, nr.y, nr.z, nr.w};
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kTetSweepThreads, 2) tet_sweep_kernel(TetArgs 
             // so the neighbour loads need not wait for the record)
             const int wd = fw[a];
             if (wd < 0) continue;
-            const T ca = rec[17 + a];
+            const T ca = rec[16 + a];
             const T* src = ((wd & 1) ? prev : cur) + pop + (size_t)(wd >> 7) * 4;
             // the neighbour's values at this cell's face vertices (j != a, ascending)
             T g[4] = {T(0), T(0), T(0), T(0)};
@@ -270,6 +271,306 @@ __global__ void __launch_bounds__(kTetSweepThreads, 2) tet_sweep_kernel(TetArgs 
         }
         __syncthreads();     // the next level reads this level's cells
     }
+}
+
+// ---------------------------------------------------------------------------
+// ring sweep
+// ---------------------------------------------------------------------------
+
+// The current iterate is only ever read by the next few levels, so a block
+// keeps its last 'ring' cells (in level order) in shared memory, and nothing
+// of it goes to global memory but what other subdomains read across
+// interfaces and, in the last iterate, f^{n+1} = 2 f* - f^n itself.  What a
+// chunk of cells needs from global memory -- f^n, coefficient records, face
+// references and the interface neighbours' values -- does not depend on the
+// sweep: loader warps copy it (cp.async) kTetAhead chunks ahead, and the cell
+// ids that address it as many chunks before that, so a level costs a barrier,
+// shared-memory loads and the solves instead of a round of global loads.
+//   A solving thread takes one cell with VPT of the block's MV variables, which
+// share the record, the face references and the selection of the face's
+// vertices.  The cells of a warp are consecutive (records and iterates of odd
+// MV lie an odd number of 16-byte words apart: no bank conflicts), and the host
+// orders a level by inflow faces, so that a warp's cells mostly take the same.
+//   Measured, 32^3 cubes x 6, D3Q4, FP32, 64 subdomains: 171 us per sweep with
+// the iterate in global memory, 81 us here (170 MB read).  What bounds it: with
+// the solves taken out a sweep takes 46 us, with the copies taken out 68 us, with
+// both out 16 us (loop and barriers): the levels' own latency, at two blocks
+// of a few warps per SM.
+template <typename T>
+__host__ __device__ constexpr size_t tet_stage_bytes(int chunk, int mv)
+{
+    // records, f^n, interface values, face references, cell ids (of this chunk,
+    // and of the cells and interface cells to copy later)
+    return (size_t)chunk * (kTetRec * sizeof(T) + 2 * (size_t)mv * 4 * sizeof(T) + 16 + 3 * 4);
+}
+
+// 4 values, shared-memory destination
+template <typename T>
+__device__ __forceinline__ void tet_cp4(T* d, const T* s)
+{
+    cp16_g2s(d, s);
+    if constexpr (sizeof(T) == 8) cp16_g2s(d + 2, s + 2);
+}
+
+template <int MV, int VPT, typename T>
+__global__ void __launch_bounds__(kTetRingThreads)
+    tet_ring_kernel(const __grid_constant__ TetArgs A, const T* __restrict__ prev, T* __restrict__ cur, int final,
+                    int whole)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    constexpr int NST = kTetAhead + 1;
+    const int s = blockIdx.x, k = blockIdx.y, C = A.plan.chunk, R = A.plan.ring;
+    const int v0 = blockIdx.z * MV, mvb = min(MV, A.m - v0);
+    const int lb = A.lstart[k * (A.nsub + 1) + s], le = A.lstart[k * (A.nsub + 1) + s + 1];
+    if (lb >= le) return;
+    const long long nodes = A.nodes;
+    const int* __restrict__ order = A.order + (size_t)k * A.ncells;
+    const long long pop = (long long)(k * A.m + v0) * nodes;
+    T* const fp = static_cast<T*>(A.f) + pop;
+    T* const ring = reinterpret_cast<T*>(smem_raw);                     // [slot][MV][4]
+    int2* const cb = reinterpret_cast<int2*>(smem_raw + (size_t)MV * R * 4 * sizeof(T));   // chunk starts
+    unsigned char* const stage0 = reinterpret_cast<unsigned char*>(cb) + 16 * (size_t)A.plan.desc;
+    const size_t stride = tet_stage_bytes<T>(C, MV);
+    auto st_rec = [&](int q) { return reinterpret_cast<T*>(stage0 + (size_t)q * stride); };
+    auto st_fn = [&](int q) { return st_rec(q) + (size_t)C * kTetRec; };        // [cell][MV][4]
+    auto st_halo = [&](int q) { return st_fn(q) + (size_t)MV * C * 4; };         // [place][MV][4]
+    auto st_ref = [&](int q) { return reinterpret_cast<int4*>(st_halo(q) + (size_t)MV * C * 4); };
+    auto st_id = [&](int q) { return reinterpret_cast<int*>(st_ref(q) + C); };
+    auto st_want = [&](int q) { return st_id(q) + C; };                          // [cell, interface cell][C]
+    const int nch = le - lb;
+    for (int e = threadIdx.x; e <= nch; e += blockDim.x) cb[e] = make_int2(A.bounds[lb + e], A.hstart[lb + e]);
+    __syncthreads();
+
+    constexpr int VG = (MV + VPT - 1) / VPT;          // solving threads per cell
+    if ((int)threadIdx.x >= VG * C) {
+        // ---- loaders ----
+        const int i = threadIdx.x - VG * C, nl = blockDim.x - VG * C;
+        const int* __restrict__ fref = A.fref + (size_t)k * A.ncells * 4;
+        const T* __restrict__ coef = static_cast<const T*>(A.coef) + (size_t)k * A.ncells * kTetRec;
+        const T* const pp = prev + pop;
+        // The ids of a chunk's cells come from global memory too: they are
+        // copied kTetAhead chunks before the chunk's data, by the thread that
+        // will use them (its own wait makes them visible to it).
+        auto fetch_ids = [&](int ch, int q) {
+            if (ch < nch) {
+                const int2 c0 = cb[ch], c1 = cb[ch + 1];
+                if (i < c1.x - c0.x) cp_small_g2s<4>(st_want(q) + i, order + c0.x + i);
+                if (i < c1.y - c0.y) cp_small_g2s<4>(st_want(q) + C + i, A.hcell + c0.y + i);
+            }
+        };
+        auto fetch = [&](int ch, int q) {
+            if (ch < nch) {
+                constexpr int RW = kTetRec * (int)sizeof(T) / 16;         // 16-byte words per record
+                const int2 c0 = cb[ch], c1 = cb[ch + 1];
+                const int p0 = c0.x, nc = c1.x - p0;
+                const T* src = coef + (size_t)p0 * kTetRec;
+                T* dst = st_rec(q);
+                for (int e = i; e < nc * RW; e += nl)
+                    cp16_g2s(dst + e * (16 / (int)sizeof(T)), src + e * (16 / (int)sizeof(T)));
+                if (i < nc) {
+                    const int id = st_want(q)[i];
+                    cp16_g2s(st_ref(q) + i, fref + (size_t)(p0 + i) * 4);
+                    st_id(q)[i] = id;
+                    T* d = st_fn(q) + i * MV * 4;
+                    const T* g = fp + (size_t)(id & (kTetOutFace - 1)) * 4;
+#pragma unroll
+                    for (int v = 0; v < MV; ++v)
+                        if (v < mvb) tet_cp4(d + v * 4, g + v * nodes);
+                }
+                if (i < c1.y - c0.y) {
+                    T* d = st_halo(q) + i * MV * 4;
+                    const T* g = pp + (size_t)st_want(q)[C + i] * 4;
+#pragma unroll
+                    for (int v = 0; v < MV; ++v)
+                        if (v < mvb) tet_cp4(d + v * 4, g + v * nodes);
+                }
+            }
+        };
+        // groups: the ids of chunks 0 .. kTetAhead - 1; then one per chunk j,
+        // with its data and the ids of chunk j + kTetAhead (into the slot that
+        // chunk j's ids leave free one step later: NST slots suffice for ids
+        // in flight as they do for data)
+        for (int j = 0; j < kTetAhead; ++j) fetch_ids(j, j);
+        cp_commit();
+        cp_wait_group<0>();
+        int q = 0, qi = kTetAhead;
+        for (int j = 0; j < kTetAhead; ++j) {
+            fetch(j, q);
+            fetch_ids(j + kTetAhead, qi);
+            cp_commit();
+            q = q == NST - 1 ? 0 : q + 1;
+            qi = qi == NST - 1 ? 0 : qi + 1;
+        }
+        cp_wait_group<kTetAhead - 1>();
+        __syncthreads();
+        for (int ch = 0; ch < nch; ++ch) {
+            fetch(ch + kTetAhead, q);
+            fetch_ids(ch + 2 * kTetAhead, qi);
+            cp_commit();
+            cp_wait_group<kTetAhead - 1>();
+            __syncthreads();          // chunk ch + 1 has landed; chunk ch is solved
+            q = q == NST - 1 ? 0 : q + 1;
+            qi = qi == NST - 1 ? 0 : qi + 1;
+        }
+        return;
+    }
+    // ---- solvers ----
+    const int vg = threadIdx.x / C, i = threadIdx.x - vg * C;
+    int slot0 = 0, q = 0;
+    __syncthreads();
+    for (int ch = 0; ch < nch; ++ch) {
+        const int nc = cb[ch + 1].x - cb[ch].x;
+        if (i < nc) {
+            const int word = st_id(q)[i];
+            const int4 nr = st_ref(q)[i];
+            const int fw[4] = {nr.x, nr.y, nr.z, nr.w};
+            const T* const halo = st_halo(q);
+            // every load before the first use (the block has few warps, and each
+            // waits out its own latencies)
+            T nb[4][VPT][4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int v = 0; v < VPT; ++v)
+                    if (fw[a] >= 0 && (MV % VPT == 0 || vg * VPT + v < MV))
+                        load4(((fw[a] & 1) ? halo : ring) + ((fw[a] >> 7) * MV + vg * VPT + v) * 4, nb[a][v]);
+            const T* const fn = st_fn(q) + (i * MV + vg * VPT) * 4;
+            T u[VPT][4], rhs[VPT][4], rec[kTetRec];
+#pragma unroll
+            for (int v = 0; v < VPT; ++v)
+                if (MV % VPT == 0 || vg * VPT + v < MV) load4(fn + v * 4, u[v]);
+#pragma unroll
+            for (int e = 0; e < kTetRec; e += 4) {
+                T r4[4];
+                load4(st_rec(q) + i * kTetRec + e, r4);
+#pragma unroll
+                for (int b = 0; b < 4; ++b) rec[e + b] = r4[b];
+            }
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                T du[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) du[b] = u[v][b] - u[v][0];
+                const T sum = (du[1] + du[2]) + du[3];
+                rhs[v][0] = sum;
+#pragma unroll
+                for (int b = 1; b < 4; ++b) rhs[v][b] = sum + du[b];
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int wd = fw[a];
+                if (wd < 0) continue;
+                // the neighbour's values at this cell's face vertices (j != a, ascending)
+#pragma unroll
+                for (int v = 0; v < VPT; ++v) {
+                    T g[3];
+#pragma unroll
+                    for (int jj = 0; jj < 3; ++jj) {
+                        const T* const nv = nb[a][v];
+                        const T lo = (wd & (1 << (5 - 2 * jj))) ? nv[1] : nv[0];
+                        const T hi = (wd & (1 << (5 - 2 * jj))) ? nv[3] : nv[2];
+                        g[jj] = ((wd & (2 << (5 - 2 * jj))) ? hi : lo) - u[v][0];
+                    }
+                    const T gs = (g[0] + g[1]) + g[2];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if (b != a) rhs[v][b] = fma(rec[16 + a], gs + g[b < a ? b : b - 1], rhs[v][b]);
+                }
+            }
+            int slot = slot0 + i;
+            if (slot >= R) slot -= R;
+            const size_t c4 = (size_t)(word & (kTetOutFace - 1)) * 4;
+            const bool send = whole || (word & kTetOutFace);
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                if (MV % VPT != 0 && vg * VPT + v >= MV) break;
+                T x[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    T acc = rec[b * 4] * rhs[v][0];
+#pragma unroll
+                    for (int j = 1; j < 4; ++j) acc = fma(rec[b * 4 + j], rhs[v][j], acc);
+                    x[b] = acc + u[v][0];
+                }
+                store4(ring + (slot * MV + vg * VPT + v) * 4, x);
+                if (vg * VPT + v >= mvb) continue;
+                if (final) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) x[b] = fma(T(2), x[b], -u[v][b]);
+                    store4(fp + (vg * VPT + v) * nodes + c4, x);
+                } else if (send) {
+                    store4(cur + pop + (vg * VPT + v) * nodes + c4, x);
+                }
+            }
+        }
+        __syncthreads();              // chunk ch is solved; chunk ch + 1 has landed
+        slot0 += nc;
+        if (slot0 >= R) slot0 -= R;
+        q = q == NST - 1 ? 0 : q + 1;
+    }
+}
+
+template <typename T>
+static const void* tet_ring_fn(int mv, int vpt)
+{
+    if (mv == 1 && vpt == 1) return (const void*)tet_ring_kernel<1, 1, T>;
+    if constexpr (sizeof(T) == 4) {
+        if (mv == 2 && vpt == 2) return (const void*)tet_ring_kernel<2, 2, T>;
+        if (mv == 3 && vpt == 2) return (const void*)tet_ring_kernel<3, 2, T>;
+        if (mv == 5 && vpt == 2) return (const void*)tet_ring_kernel<5, 2, T>;
+        if (mv == 6 && vpt == 2) return (const void*)tet_ring_kernel<6, 2, T>;
+    }
+    return nullptr;
+}
+
+// The shape of a ring sweep.  One block per (subdomain, velocity) when those
+// fill the SMs, so that the m variables share the records; else the variables
+// are split over blocks.  Chunks as wide as the thread limit, the widest level
+// and shared memory allow, where two blocks per SM (113 KB each) go before
+// wider chunks when there are blocks for both: a block waits for its own
+// latencies most of the time (32^3 cubes x 6, D3Q4, FP32: 64 cells and two
+// blocks 4.14 ms per 15 steps, 96 cells and one block 5.17 ms).  Two variables
+// per solving thread measured best of 1, 2 and 3 (5.23, 4.26, 20 ms: three
+// spill).  FP64 always splits the variables: its solves are bound by the FP64
+// units, not by the records' traffic (21^3 cubes, D3Q6 Euler, 8 steps: 8.3 ms
+// together, 5.2 split; global iterate 8.2).  Warps are solvers or loaders as a whole: chunks are multiples of 32.
+bool tet_make_plan(int ring, int width, int levels, int cells, int blocks, int m, int prec, TetPlan* plan)
+{
+    const size_t es = prec == 1 ? 4 : 8;
+    for (int groups = 1; groups <= m; ++groups) {
+        const int mv = (m + groups - 1) / groups;
+        if ((m + mv - 1) / mv != groups) continue;             // the same split as fewer groups
+        if (groups < m && ((long long)blocks * groups < 152 || prec == 0)) continue;
+        const int vpt = std::min(mv, 2), vg = (mv + vpt - 1) / vpt;
+        const int cmax = std::min(kTetRingThreads / (vg + 1) / 32 * 32, (width + 31) / 32 * 32);
+        const bool two = (long long)blocks * groups > 152;
+        for (int pass = two ? 0 : 1; pass < 2; ++pass)
+            for (int c = cmax; c >= 32; c -= 32) {
+                if (pass == 0 && c < std::min(64, cmax)) break;
+                const size_t stage = prec == 1 ? tet_stage_bytes<float>(c, mv) : tet_stage_bytes<double>(c, mv);
+                // chunks of a subdomain at most: one per level, one per c cells, one per
+                // c interface cells (3 per cell at most); two chunk starts per 16 bytes
+                const int desc = (levels + 4 * (cells / c + 1) + 2) / 2;
+                const size_t sm = (size_t)mv * ring * 4 * es + 16 * (size_t)desc + (kTetAhead + 1) * stage;
+                if (sm > (pass == 0 ? 113 : 227) * 1024) continue;
+                plan->chunk = c;
+                plan->mv = mv;
+                plan->vpt = vpt;
+                plan->groups = groups;
+                plan->ring = ring;
+                plan->desc = desc;
+                plan->threads = c * (vg + 1);
+                plan->smem = sm;
+                return true;
+            }
+    }
+    return false;
+}
+
+cudaError_t tet_configure(const TetPlan& plan, int prec)
+{
+    const void* fn = prec == 1 ? tet_ring_fn<float>(plan.mv, plan.vpt) : tet_ring_fn<double>(plan.mv, plan.vpt);
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 // ---------------------------------------------------------------------------
@@ -333,12 +634,12 @@ __device__ __forceinline__ void tet_equilibria(const TetArgs& A, const V* W, V* 
     }
 }
 
-// f^{n+1} = 2 f* - f^n, then W = sum_k f_k (Kahan in FP32) and the
-// relaxation f <- omega M(W) + (1 - omega) f (eq. over_relaxation); Maxwell
+// f^{n+1} = 2 f* - f^n (EXTRAP; else f holds f^{n+1}: the ring sweep writes
+// it), then W = sum_k f_k (Kahan in FP32) and the relaxation f <- omega M(W) + (1 - omega) f (eq. over_relaxation); Maxwell
 // with conductivity relaxes about the equilibrium after the source step,
 // f <- M(W+) + (1 - omega)(f - M(W-)).  Compiled per system and velocity
 // set, so that every population stays in registers.
-template <int SYS, int VS, typename T>
+template <int SYS, int VS, bool EXTRAP, typename T>
 __global__ void __launch_bounds__(256) tet_relax_kernel(TetArgs A, const T* __restrict__ star)
 {
     constexpr int m = nvars(3, SYS), NV = VS == 1 ? 4 : 6, NPOP = NV * m;
@@ -348,7 +649,10 @@ __global__ void __launch_bounds__(256) tet_relax_kernel(TetArgs A, const T* __re
          i += (long long)gridDim.x * blockDim.x) {
         T fk[NPOP];
 #pragma unroll
-        for (int p = 0; p < NPOP; ++p) fk[p] = fma(T(2), star[p * nodes + i], -f[p * nodes + i]);
+        for (int p = 0; p < NPOP; ++p) {
+            fk[p] = f[p * nodes + i];
+            if (EXTRAP) fk[p] = fma(T(2), star[p * nodes + i], -fk[p]);
+        }
         T W[m];
 #pragma unroll
         for (int v = 0; v < m; ++v) {
@@ -448,7 +752,8 @@ template <int S, int V, typename T>
 struct RelaxLaunch {
     static void launch(const TetArgs& a, unsigned grid, cudaStream_t st, const void* star)
     {
-        tet_relax_kernel<S, V, T><<<grid, 256, 0, st>>>(a, static_cast<const T*>(star));
+        if (star) tet_relax_kernel<S, V, true, T><<<grid, 256, 0, st>>>(a, static_cast<const T*>(star));
+        else tet_relax_kernel<S, V, false, T><<<grid, 256, 0, st>>>(a, nullptr);
     }
 };
 
@@ -468,8 +773,14 @@ cudaError_t tet_launch_setup(const TetSetupArgs& a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t tet_launch_sweep(const TetArgs& a, const void* prev, void* cur, int prec, cudaStream_t st)
+cudaError_t tet_launch_sweep(const TetArgs& a, const void* prev, void* cur, int final, int whole, int prec,
+                             cudaStream_t st)
 {
+    if (a.plan.chunk > 0) {
+        void* args[] = {(void*)&a, (void*)&prev, (void*)&cur, (void*)&final, (void*)&whole};
+        return cudaLaunchKernel(prec == 1 ? tet_ring_fn<float>(a.plan.mv, a.plan.vpt) : tet_ring_fn<double>(a.plan.mv, a.plan.vpt),
+                                dim3(a.nsub, a.nvel, a.plan.groups), dim3(a.plan.threads), args, a.plan.smem, st);
+    }
     const dim3 grid(a.nsub, a.nvel);
     if (prec == 1)
         tet_sweep_kernel<float><<<grid, kTetSweepThreads, 0, st>>>(a, static_cast<const float*>(prev),
