@@ -179,24 +179,12 @@ static int next_divisor_below(int L, int b)
     return 1;
 }
 
-// Default cell block: start from the whole subdomain and shrink the longest
-// extent (z before y before x on ties, to keep the contiguous x rows long)
-// until one tile fits the shared-memory target -- two tiles then fit twice
-// per SM -- and the grid has enough tiles to fill 152 SMs twice.
-static void choose_block(const kin_ctx* c, int B[3])
+// Cell block of the generic kernel by shrinking the whole subdomain: the
+// longest extent first (z before y before x on ties, to keep the contiguous x
+// rows long) until one tile fits 48 KB and the grid has enough tiles to fill
+// 152 SMs twice.
+static void shrink_block(const kin_ctx* c, int B[3])
 {
-    // a block shape with a compiled fixed-shape kernel, if one fits the subdomains
-    int shapes[4][3];
-    const int ns = fixed_shapes(c->dim, c->degree, c->system, c->precision, shapes);
-    for (int k = 0; k < ns; ++k) {
-        bool fits = true;
-        for (int a = 0; a < 3; ++a)
-            if (c->L[a] % shapes[k][a]) fits = false;
-        if (fits) {
-            for (int a = 0; a < 3; ++a) B[a] = shapes[k][a];
-            return;
-        }
-    }
     const size_t target = 48 * 1024;
     for (int a = 0; a < 3; ++a) B[a] = c->L[a];
     auto grid_of = [&](const int* b) {
@@ -215,6 +203,78 @@ static void choose_block(const kin_ctx* c, int B[3])
         if (!too_big && B[best] <= 4) break;     // keep lines reasonably long
         B[best] = next_divisor_below(c->L[best], B[best]);
     }
+}
+
+// Default cell block: a shape with a compiled fixed-shape kernel if one fits
+// the subdomains; else the divisors of the subdomain extents for which the
+// generic kernel is estimated to be fastest.
+//   Instructions per value: the relaxation and the sweep's arithmetic; the row
+// copies, whose decode is shared by a row; and per line of B cells its
+// look-back (the block summaries above rounding, about 26 cells back at the
+// usual time steps, at most the K - 1 subdomains) and the set-up of its sweep and
+// summary, shared by its B (p + 1) values.  Thin blocks, which is what shrinking
+// leaves of extents like 25 or 29, cost several times the rest.
+//   Time: a tile's phases take about 10,000 cycles of latency whatever its
+// size, shared by the tiles resident on an SM, plus their instructions.
+//   290 x 210 cells, p = 1, subdomains of 29 x 35: 130 us per step with the
+// shrunk 1 x 7 blocks, 22 us with 29 x 5.  A block never needs more summary
+// memory than the shrunk one (its thinnest extent is no smaller).
+static void choose_block(const kin_ctx* c, int B[3])
+{
+    int shapes[4][3];
+    const int ns = fixed_shapes(c->dim, c->degree, c->system, c->precision, shapes);
+    for (int k = 0; k < ns; ++k) {
+        bool fits = true;
+        for (int a = 0; a < 3; ++a)
+            if (c->L[a] % shapes[k][a]) fits = false;
+        if (fits) {
+            for (int a = 0; a < 3; ++a) B[a] = shapes[k][a];
+            return;
+        }
+    }
+    shrink_block(c, B);
+    if (c->dim < 2) return;
+    int least = B[0];
+    for (int a = 1; a < c->dim; ++a) least = std::min(least, B[a]);
+    std::vector<int> div[3];
+    for (int a = 0; a < 3; ++a)
+        for (int d = a < c->dim ? least : 1; d <= c->L[a]; ++d)
+            if (c->L[a] % d == 0) div[a].push_back(d);
+    double best = 0.0;
+    for (int b0 : div[0])
+        for (int b1 : div[1])
+            for (int b2 : div[2]) {
+                const int b[3] = {b0, b1, b2};
+                const double cells = (double)b0 * b1 * b2;
+                if (cells * c->npop * c->NN * c->esize > 227 * 1024) continue;
+                const int rowlen = b0 * c->NN;
+                const int wide = rowlen * c->esize % 16 == 0 ? (int)(16 / c->esize) : 1, words = rowlen / wide;
+                int lanes = 2;
+                while (lanes < 32 && lanes < words) lanes *= 2;
+                double instr = 25.0 + 2.0 * lanes * (25.0 + 6.0 * ((words + lanes - 1) / lanes)) / rowlen;
+                double items = 0, tiles = 1;
+                for (int a = 0; a < c->dim; ++a) {
+                    const double nb = (double)c->L[a] / b[a];
+                    const double folds = std::min((c->iters - 0.5) * nb, std::ceil(26.0 / b[a]));
+                    instr += (100.0 + 8.0 * folds) / (b[a] * c->NP);
+                    items += 2.0 * c->m * (cells / b[a]) * (c->NN / c->NP);
+                    tiles *= c->n[a] / b[a];
+                }
+                const double values = cells * c->npop * c->NN;
+                const double sm = values * c->esize + items * c->esize + 1024;
+                if (sm > 228.0 * 1024) continue;
+                // warp instructions at 60% of the issue rate, less when fewer
+                // than four tiles share the SM; the FP64 units add about 5 cycles a value
+                const double per_sm = std::min(8.0, std::floor(228.0 * 1024 / sm));
+                const double resident = tiles / (152.0 * std::max(1.0, tiles / (152.0 * per_sm) + 0.3));
+                const double shared = std::max(1.0, resident);
+                const double w = instr / 77.0 / std::min(1.0, shared / 4.0) + (c->esize == 8 ? 5.0 : 0.0);
+                const double rate = resident * values / (10000.0 + shared * values * w);
+                if (rate > best) {
+                    best = rate;
+                    for (int a = 0; a < 3; ++a) B[a] = b[a];
+                }
+            }
 }
 
 // Bulk copies need every row of a cell block to start on a 16-byte
@@ -268,7 +328,9 @@ static Inst make_inst(const kin_ctx* c, int mode)
     I.fd_rowlen = make_fastdiv((unsigned)(c->B[0] * c->NN));
     I.iters = c->iters;
     I.mode = mode;
-    I.tma = rows_are_16b_aligned(c) ? 1 : 0;
+    I.vec = rows_are_16b_aligned(c) ? 1 : 0;
+    // (the bounded-wait test hook lives in the bulk-copy path)
+    I.tma = I.vec && (c->stages == 2 || (c->debug_flags & KIN_DEBUG_STALL_LOAD)) ? 1 : 0;
     I.stages = c->stages;
     I.debug_stall = (c->debug_flags & KIN_DEBUG_STALL_LOAD) ? 1 : 0;
     I.lambda = c->lambda;

@@ -189,6 +189,10 @@ int mixed_kernels_2d(MixedKernel* out, int max);
 // shared-memory tile buffers, or fn == nullptr.
 FixedKernel fixed_kernel_d2(int degree, int system, int prec, const int B[3], int stages);
 FixedKernel fixed_kernel_d3(int degree, int system, int prec, const int B[3], int stages);
+// The same for the shapes of kin_step_hi.cu (FP32, 3D degrees 2 and 3) and
+// kin_step_f64.cu; one tile buffer, no batched kernel.
+FixedKernel fixed_kernel_hi(int dim, int degree, int system, const int B[3]);
+FixedKernel fixed_kernel_f64(int dim, int degree, int system, const int B[3]);
 // Tile buffers the fixed-shape kernel of a shape uses unless asked otherwise.
 int fixed_default_stages(int dim, int degree, int system, int prec, const int B[3]);
 // Preferred fixed block shapes for a (dim, degree, system, precision), best first;

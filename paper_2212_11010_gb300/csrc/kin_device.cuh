@@ -98,6 +98,7 @@ struct __align__(16) Inst {
     int iters;               // K
     int mode;                // 0: full step, 1: summaries only (no transport, no store)
     int tma;                 // 1: rows moved by bulk copies (alignment checked on the host)
+    int vec;                 // 1: every row is whole, aligned 16-byte words
     int stages;              // shared-memory tile buffers per thread block (1 or 2)
     int debug_stall;         // test hook: the load barrier expects 16 bytes that never arrive
     double lambda, gamma, omega;
@@ -613,27 +614,50 @@ __device__ __forceinline__ void issue_tile_store(const Inst& I, int t, const T* 
     bulk_commit();
 }
 
-// Element-wise load / store of a tile (used when rows are not 16-byte aligned).
-template <int D, int P, int SYS, typename T, bool LOAD>
-__device__ __forceinline__ void copy_tile_generic(const Inst& I, int t, T* s)
+// Load / store of a tile through the load/store units, in words of N elements
+// (16 bytes where every row is whole words, else one element): 'lanes' lanes
+// per row, the power of two that covers it in the fewest steps, so that a row
+// is decoded once (two divisions per element took two thirds of the
+// instructions before).  cp.async stages nothing in registers; the loads are
+// waited for here, and the caller's barrier shows them to the block.
+template <int D, int P, int SYS, typename T, bool LOAD, int N>
+__device__ __forceinline__ void copy_rows(const Inst& I, int t, T* s)
 {
     constexpr int NN = ipow(P + 1, D);
     constexpr int NPOP = 2 * D * (nvars(D, SYS));
     const int B0 = I.B[0], B1 = D > 1 ? I.B[1] : 1, B2 = D > 2 ? I.B[2] : 1;
-    const int bcells = B0 * B1 * B2, rowlen = B0 * NN, nrows = B1 * B2;
-    const int nload = NPOP * nrows * rowlen;
+    const int bcells = B0 * B1 * B2, rowlen = B0 * NN, nrows = B1 * B2, nchunks = NPOP * nrows;
     const TileXYZ c = tile_xyz(I, t);
     T* f = static_cast<T*>(I.f);
-    for (int idx = threadIdx.x; idx < nload; idx += blockDim.x) {
-        const int ch = (int)fdiv((unsigned)idx, I.fd_rowlen);
-        const int e = idx - ch * rowlen;
+    const int words = rowlen / N;
+    const int sh = words > 16 ? 5 : (words > 8 ? 4 : (words > 4 ? 3 : (words > 2 ? 2 : 1)));
+    const int e0 = threadIdx.x & ((1 << sh) - 1);
+    for (int ch = threadIdx.x >> sh; ch < nchunks; ch += blockDim.x >> sh) {
         const int pop = (int)fdiv((unsigned)ch, I.fd_nrows);
         const int row = ch - pop * nrows;
-        const long long g = row_offset<D, NN>(I, pop, row, c.bx * B0, c.by * B1, c.bz * B2) + e;
-        T& sv = s[(pop * bcells + row * B0) * NN + e];
-        if (LOAD) sv = f[g];
-        else f[g] = sv;
+        T* g = f + row_offset<D, NN>(I, pop, row, c.bx * B0, c.by * B1, c.bz * B2);
+        T* sv = s + (pop * bcells + row * B0) * NN;
+        for (int e = e0; e < words; e += 1 << sh) {
+            if constexpr (N > 1) {
+                if (LOAD) cp16_g2s(sv + e * N, g + e * N);
+                else *reinterpret_cast<uint4*>(g + e * N) = *reinterpret_cast<const uint4*>(sv + e * N);
+            } else {
+                if (LOAD) cp_small_g2s<sizeof(T)>(sv + e, g + e);
+                else g[e] = sv[e];
+            }
+        }
     }
+    if (LOAD) {
+        cp_commit();
+        cp_wait_all();
+    }
+}
+
+template <int D, int P, int SYS, typename T, bool LOAD>
+__device__ __forceinline__ void copy_tile_generic(const Inst& I, int t, T* s)
+{
+    if (I.vec) copy_rows<D, P, SYS, T, LOAD, 16 / (int)sizeof(T)>(I, t, s);
+    else copy_rows<D, P, SYS, T, LOAD, 1>(I, t, s);
 }
 
 // Phases 2-4 on a loaded tile; ends after the summaries (no trailing barrier).
@@ -660,9 +684,9 @@ __device__ __forceinline__ void chain_tile(const Inst& I, int t, T* tin)
 }
 
 // Persistent step kernel: each thread block walks the tiles blockIdx.x,
-// blockIdx.x + gridDim.x, ...  With bulk copies and two shared-memory stages
-// the load of the next tile and the store of the previous one run while the
-// current tile is computed.
+// blockIdx.x + gridDim.x, ...  With two shared-memory stages rows move by bulk
+// copies, and the load of the next tile and the store of the previous one run
+// while the current tile is computed; with one, through the load/store units.
 template <int D, int P, int SYS, typename T>
 __global__ void __launch_bounds__(kThreads) step_kernel(const __grid_constant__ Inst I)
 {

@@ -19,6 +19,7 @@ static StepKernel pick(int prec)
 #define KIN_FIXED_2D(X)                           \
     X(1, kEuler, float, 16, 8, 128, 6, 3)         \
     X(1, kEuler, float, 16, 16, 256, 3, 1)        \
+    X(1, kEuler, float, 8, 8, 128, 6, 3)          \
     X(2, kEuler, float, 8, 8, 192, 5, 3)          \
     X(3, kEuler, float, 8, 4, 128, 6, 3)          \
     X(3, kEuler, float, 8, 8, 256, 3, 1)          \
@@ -44,6 +45,7 @@ FixedKernel fixed_kernel_d2(int degree, int system, int prec, const int B[3], in
     }
     KIN_FIXED_2D(KIN_TRY)
 #undef KIN_TRY
+    if (stages == 1 && prec == 0) return fixed_kernel_f64(2, degree, system, B);
     return k;
 }
 

@@ -47,6 +47,7 @@ FixedKernel fixed_kernel_d3(int degree, int system, int prec, const int B[3], in
     }
     KIN_FIXED_3D(KIN_TRY)
 #undef KIN_TRY
+    if (stages == 1) return prec == 1 ? fixed_kernel_hi(3, degree, system, B) : fixed_kernel_f64(3, degree, system, B);
     return k;
 }
 
@@ -66,20 +67,12 @@ int fixed_shapes(int dim, int degree, int system, int prec, int out[4][3])
             ++n;
         }
     };
-    if (system == kMaxwell) {
-        if (dim == 3 && prec == 1 && degree == 1) {
-            add(4, 4, 4);
-            add(4, 4, 2);
-            add(8, 2, 2);
-            add(4, 2, 2);
-        }
-        return n;
-    }
-    if (system != kEuler) return 0;
+    if (system == kAdvection || (system == kMaxwell && dim != 3)) return 0;
     if (dim == 2 && prec == 1) {
         if (degree == 1) {
             add(16, 16, 1);
             add(16, 8, 1);
+            add(8, 8, 1);
         }
         if (degree == 2) add(8, 8, 1);
         if (degree == 3) {
@@ -87,12 +80,20 @@ int fixed_shapes(int dim, int degree, int system, int prec, int out[4][3])
             add(8, 4, 1);
         }
     }
-    if (dim == 2 && prec == 0 && degree == 2) add(8, 8, 1);
+    if (dim == 2 && prec == 0) degree == 3 ? add(8, 4, 1) : add(8, 8, 1);
     if (dim == 3 && prec == 1 && degree == 1) {
         add(4, 4, 4);
-        add(8, 4, 2);
+        if (system == kEuler) add(8, 4, 2);
         add(4, 4, 2);
         add(8, 2, 2);
+        if (system == kMaxwell) add(4, 2, 2);
+    }
+    if (dim == 3 && prec == 1 && degree == 2) add(4, 2, 2);
+    if (dim == 3 && prec == 1 && degree == 3) add(2, 2, 2);
+    if (dim == 3 && prec == 0) {
+        if (degree == 1) add(4, 4, 2);
+        if (degree == 2) add(2, 2, 2);
+        if (degree == 3) add(2, 2, 1);
     }
     return n;
 }
