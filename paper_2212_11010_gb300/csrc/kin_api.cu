@@ -74,7 +74,6 @@ struct kin_ctx {
     // tetrahedral meshes
     bool tet = false;
     int nsub = 0;
-    int tsgn[4][3] = {};
     void* tcoef = nullptr;            // T records [velocity][cell][kTetRec]
     int* torder = nullptr;            // [velocity][cells]
     int* tlstart = nullptr;           // [velocity][nsub + 1]
@@ -287,6 +286,12 @@ static bool rows_are_16b_aligned(const kin_ctx* c)
     return rowb % 16 == 0 && popb % 16 == 0 && lineb % 16 == 0 && ((uintptr_t)c->f % 16) == 0;
 }
 
+static RelaxConsts relax_constants(const kin_ctx* c)
+{
+    const double mu = c->system == KIN_MAXWELL ? (1.0 - 0.5 * c->sigma * c->dt) / (1.0 + 0.5 * c->sigma * c->dt) : 1.0;
+    return relax_consts(c->lambda, c->gamma, c->omega, mu, c->adv);
+}
+
 static Inst make_inst(const kin_ctx* c, int mode)
 {
     Inst I;
@@ -315,7 +320,6 @@ static Inst make_inst(const kin_ctx* c, int mode)
         I.nblk[a] = c->nblk[a];
         I.nb[a] = c->nb[a];
         I.NS[a] = c->tiles[a];
-        I.adv[a] = c->adv[a];
         I.ax[a].lines = make_fastdiv((unsigned)((bcells / c->B[a]) * tn));
         I.ax[a].e1 = make_fastdiv((unsigned)(a == 0 ? c->B[1] : c->B[0]));
         I.ax[a].glines = (long long)(c->cells / c->n[a]) * tn;
@@ -333,10 +337,7 @@ static Inst make_inst(const kin_ctx* c, int mode)
     I.tma = I.vec && (c->stages == 2 || (c->debug_flags & KIN_DEBUG_STALL_LOAD)) ? 1 : 0;
     I.stages = c->stages;
     I.debug_stall = (c->debug_flags & KIN_DEBUG_STALL_LOAD) ? 1 : 0;
-    I.lambda = c->lambda;
-    I.gamma = c->gamma;
-    I.omega = c->omega;
-    I.mu = c->system == KIN_MAXWELL ? (1.0 - 0.5 * c->sigma * c->dt) / (1.0 + 0.5 * c->sigma * c->dt) : 1.0;
+    I.rx = relax_constants(c);
     for (int a = 0; a < 3; ++a) I.inflow[a] = c->inflow[a];
     I.bnd = c->bnd_dev;
     // look-back depth per direction: the fewest upstream blocks d with
@@ -539,9 +540,12 @@ static SxArgs sx_args(const kin_ctx* c)
     S.npop = c->npop;
     S.system = c->system;
     S.lambda = c->lambda;
-    S.omega = c->omega;
     S.gamma = c->gamma;
-    for (int i = 0; i < 16; ++i) S.minv[i] = c->minv[i];
+    S.rx = relax_constants(c);
+    for (int i = 0; i < 16; ++i) {
+        S.minv[i] = c->minv[i];
+        S.minvf[i] = (float)c->minv[i];
+    }
     long long total = 0;
     for (int pop = 0; pop < c->npop; ++pop)
         for (int a = 0; a < c->dim; ++a)
@@ -598,11 +602,8 @@ static TetArgs tet_args(const kin_ctx* c)
     a.f = c->f;
     a.lambda = c->lambda;
     a.gamma = c->gamma;
-    a.omega = c->omega;
-    a.mu = c->system == KIN_MAXWELL ? (1.0 - 0.5 * c->sigma * c->dt) / (1.0 + 0.5 * c->sigma * c->dt) : 1.0;
+    a.rx = relax_constants(c);
     for (int i = 0; i < 3; ++i) a.adv[i] = c->adv[i];
-    for (int k = 0; k < 4; ++k)
-        for (int i = 0; i < 3; ++i) a.sgn[k][i] = c->tsgn[k][i];
     return a;
 }
 
@@ -1050,7 +1051,6 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
     for (int k = 0; k < c->nvel; ++k)
         for (int a = 0; a < 3; ++a) {
             if (c->simplex) {
-                c->tsgn[k][a] = s3[k][a];
                 vel[k][a] = c->lambda * s3[k][a];
             } else {
                 vel[k][a] = a == k / 2 ? (k % 2 ? -c->lambda : c->lambda) : 0.0;

@@ -12,6 +12,40 @@ constexpr int kDiagBlocks = 304;   // 2 x 152 SMs
 
 struct Inst;
 
+// Constants of the relaxation in both precisions, computed once on the host:
+// one FP64 operation of a warp occupies the SM's FP64 units for 16 cycles, so
+// the conversions and the division 1 / (2 lambda) at the head of every tile (or
+// thread) took up to a quarter of a kernel's time: a batch step of 24 uneven 2D
+// problems (FP32) ran 0.88 ms with them.
+template <typename T>
+struct RelaxK {
+    T omega, om1, gm1, inv2l, inv4l, mu, adv[3];     // om1 = 1 - omega, gm1 = gamma - 1, inv2l = 1 / (2 lambda)
+};
+struct RelaxConsts {
+    RelaxK<float> f;
+    RelaxK<double> d;
+    int two;                                         // omega == 2
+};
+template <typename T>
+inline void relax_consts(RelaxK<T>& k, double lambda, double gamma, double omega, double mu, const double* adv)
+{
+    k.omega = (T)omega;
+    k.om1 = T(1) - (T)omega;
+    k.gm1 = (T)(gamma - 1.0);
+    k.inv2l = (T)(1.0 / (2.0 * lambda));
+    k.inv4l = (T)(1.0 / (4.0 * lambda));
+    k.mu = (T)mu;
+    for (int a = 0; a < 3; ++a) k.adv[a] = (T)adv[a];
+}
+inline RelaxConsts relax_consts(double lambda, double gamma, double omega, double mu, const double* adv)
+{
+    RelaxConsts r;
+    relax_consts(r.f, lambda, gamma, omega, mu, adv);
+    relax_consts(r.d, lambda, gamma, omega, mu, adv);
+    r.two = omega == 2.0;
+    return r;
+}
+
 struct SetupArgs {
     int dim, degree;
     double lambda, dt;
@@ -69,9 +103,11 @@ struct SxArgs {
     int dim, degree, nn, m, nvel, npop, system;
     int from_f;                   // iterate 1: interface inflow is f^n of the upwind cell
     int final_iter;
-    double lambda, omega, gamma;
+    double lambda, gamma;
     double adv[3];
     double minv[16];
+    float minvf[16];
+    RelaxConsts rx;
 };
 
 cudaError_t sx_launch_setup(const SxSetupArgs& a, cudaStream_t st);
@@ -132,9 +168,9 @@ struct TetArgs {
     const int* hcell;
     TetPlan plan;
     void* f;                      // T [pop][cell][4]
-    double lambda, gamma, omega, mu;
+    double lambda, gamma;
     double adv[3];
-    int sgn[4][3];                // D3Q4 velocity signs
+    RelaxConsts rx;
 };
 constexpr int kTetOutFace = 1 << 30;
 

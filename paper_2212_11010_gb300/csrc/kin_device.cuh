@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "kin_aux.h"
 #include "kin_tma.cuh"
 
 namespace kin {
@@ -101,8 +102,7 @@ struct __align__(16) Inst {
     int vec;                 // 1: every row is whole, aligned 16-byte words
     int stages;              // shared-memory tile buffers per thread block (1 or 2)
     int debug_stall;         // test hook: the load barrier expects 16 bytes that never arrive
-    double lambda, gamma, omega;
-    double mu;               // Maxwell: conductivity source factor (1 - sigma dt/2) / (1 + sigma dt/2)
+    RelaxConsts rx;          // (mu, Maxwell: conductivity source factor (1 - sigma dt/2) / (1 + sigma dt/2))
     int inflow[3];           // 1: axis a has inflow boundaries instead of being periodic
     // look-back depth per (axis, sign): only the last lbdepth blocks of a walk
     // are folded; every earlier contribution reaches the inflow damped by
@@ -113,12 +113,18 @@ struct __align__(16) Inst {
     // T*: inflow boundaries: per population the value across the
     // domain-boundary face it enters through, M_k(W_b)[v] of that face's state
     const void* bnd;
-    double adv[3];
     // block-inverse coefficients (computed in FP64 on the device once per
     // context), carried in the launch parameters: read from the constant bank
     double cd[6][kCoefStride];
     float cf[6][kCoefStride];
 };
+
+template <typename T>
+__device__ __forceinline__ const RelaxK<T>& relax_k(const RelaxConsts& r)
+{
+    if constexpr (sizeof(T) == 4) return r.f;
+    else return r.d;
+}
 
 template <typename T>
 __device__ __forceinline__ const T* coef_rec(const Inst& I, int dir);
@@ -496,10 +502,9 @@ __device__ __forceinline__ void relax_block(const Inst& I, T* s, int bcells)
     constexpr int NPOP = NV * M;
     const int nnodes = bcells * NN;
     const int pstride = bcells * NN;
-    const T omega = T(I.omega);
-    const bool two = I.omega == 2.0;
-    const T inv2l = T(1.0 / (2.0 * I.lambda));
-    const T gm1 = T(I.gamma - 1.0);
+    const RelaxK<T>& RK = relax_k<T>(I.rx);
+    const T omega = RK.omega, om1 = RK.om1, inv2l = RK.inv2l, gm1 = RK.gm1;
+    const bool two = I.rx.two;
     for (int nd = threadIdx.x; nd < nnodes; nd += blockDim.x) {
         T fk[NPOP];
 #pragma unroll
@@ -513,7 +518,7 @@ __device__ __forceinline__ void relax_block(const Inst& I, T* s, int bcells)
             W[v] = acc.s;
         }
         if constexpr (SYS == kMaxwell) {
-            maxwell_relax_node(fk, W, T(I.mu), T(1) - omega, inv2l);
+            maxwell_relax_node(fk, W, RK.mu, om1, inv2l);
 #pragma unroll
             for (int pp = 0; pp < NPOP; ++pp) s[pp * pstride + nd] = fk[pp];
             continue;
@@ -530,7 +535,7 @@ __device__ __forceinline__ void relax_block(const Inst& I, T* s, int bcells)
         for (int a = 0; a < D; ++a) {
             T Q[M];
             if (SYS == kAdvection) {
-                Q[0] = T(I.adv[a]) * W[0];
+                Q[0] = RK.adv[a] * W[0];
             } else {
                 const T ua = W[1 + a] * inv;
                 Q[0] = W[1 + a];
@@ -548,8 +553,8 @@ __device__ __forceinline__ void relax_block(const Inst& I, T* s, int bcells)
                     fp = fma(T(2), base + half, -fp);
                     fm = fma(T(2), base - half, -fm);
                 } else {
-                    fp = omega * (base + half) + (T(1) - omega) * fp;
-                    fm = omega * (base - half) + (T(1) - omega) * fm;
+                    fp = omega * (base + half) + om1 * fp;
+                    fm = omega * (base - half) + om1 * fm;
                 }
             }
         }

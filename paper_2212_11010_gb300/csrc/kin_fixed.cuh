@@ -569,10 +569,9 @@ __device__ __forceinline__ void fixed_relax(const Inst& I, T* s)
 {
     using S = Shape<D, P, SYS, T, B0, B1, B2>;
     constexpr int M = S::M, NV = 2 * D, NPOP = S::NPOP;
-    const T omega = T(I.omega);
-    const bool two = I.omega == 2.0;
-    const T inv2l = T(1.0 / (2.0 * I.lambda));
-    const T gm1 = T(I.gamma - 1.0);
+    const RelaxK<T>& RK = relax_k<T>(I.rx);
+    const T omega = RK.omega, om1 = RK.om1, inv2l = RK.inv2l, gm1 = RK.gm1;
+    const bool two = I.rx.two;
 #pragma unroll
     for (int k = 0; k < (S::NODES + NTH - 1) / NTH; ++k) {
         const int nd = threadIdx.x + k * NTH;
@@ -590,7 +589,7 @@ __device__ __forceinline__ void fixed_relax(const Inst& I, T* s)
             W[v] = acc.s;
         }
         if constexpr (SYS == kMaxwell) {
-            maxwell_relax_node(fk, W, T(I.mu), T(1) - omega, inv2l);
+            maxwell_relax_node(fk, W, RK.mu, om1, inv2l);
 #pragma unroll
             for (int pp = 0; pp < NPOP; ++pp) s[pp * S::PSTR + o] = fk[pp];
             continue;
@@ -607,7 +606,7 @@ __device__ __forceinline__ void fixed_relax(const Inst& I, T* s)
         for (int a = 0; a < D; ++a) {
             T Q[M];
             if (SYS == kAdvection) {
-                Q[0] = T(I.adv[a]) * W[0];
+                Q[0] = RK.adv[a] * W[0];
             } else {
                 const T ua = W[1 + a] * inv;
                 Q[0] = W[1 + a];
@@ -625,8 +624,8 @@ __device__ __forceinline__ void fixed_relax(const Inst& I, T* s)
                     fp = fma(T(2), base + half, -fp);
                     fm = fma(T(2), base - half, -fm);
                 } else {
-                    fp = omega * (base + half) + (T(1) - omega) * fp;
-                    fm = omega * (base - half) + (T(1) - omega) * fm;
+                    fp = omega * (base + half) + om1 * fp;
+                    fm = omega * (base - half) + om1 * fm;
                 }
             }
         }
@@ -664,10 +663,9 @@ __device__ __forceinline__ void fixed_relax_pairs(const Inst& I, float* s)
     constexpr int M = S::M, NV = 2 * D, NPOP = S::NPOP;
     constexpr int NPAIR = S::NODES / 2;
     static_assert(S::ROWLEN % 2 == 0 && S::RSTR % 2 == 0 && S::PSTR % 2 == 0, "node pairs must be 8-byte words");
-    const bool two = I.omega == 2.0;
-    const float2 om = f2((float)I.omega), omc = f2(1.0f - (float)I.omega);
-    const float2 inv2l = f2((float)(1.0 / (2.0 * I.lambda)));
-    const float2 gm1 = f2((float)(I.gamma - 1.0));
+    const RelaxK<float>& RK = I.rx.f;
+    const bool two = I.rx.two;
+    const float2 om = f2(RK.omega), omc = f2(RK.om1), inv2l = f2(RK.inv2l), gm1 = f2(RK.gm1);
     const float2 twof = f2(2.0f);
 #pragma unroll
     for (int k = 0; k < (NPAIR + NTH - 1) / NTH; ++k) {
@@ -714,7 +712,7 @@ __device__ __forceinline__ void fixed_relax_pairs(const Inst& I, float* s)
         }
         if constexpr (SYS == kMaxwell) {
             // maxwell_relax_node on node pairs
-            const float2 mu = f2((float)I.mu), zero = f2(0.0f);
+            const float2 mu = f2(RK.mu), zero = f2(0.0f);
             auto neg2 = [](float2 x) { return make_float2(-x.x, -x.y); };
             float2 Wp[M];
 #pragma unroll
@@ -754,7 +752,7 @@ __device__ __forceinline__ void fixed_relax_pairs(const Inst& I, float* s)
         for (int a = 0; a < D; ++a) {
             float2 Q[M];
             if (SYS == kAdvection) {
-                Q[0] = mul2(f2((float)I.adv[a]), W[0]);
+                Q[0] = mul2(f2(RK.adv[a]), W[0]);
             } else {
                 const float2 ua = mul2(W[1 + a], inv);
                 Q[0] = W[1 + a];

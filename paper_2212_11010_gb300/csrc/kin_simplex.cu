@@ -774,18 +774,16 @@ __global__ void __launch_bounds__(MAXT) sx_wave_kernel(const __grid_constant__ S
 // Relaxation with the d + 1 velocity equilibria: M_{k,v} = sum_j Minv[k][j] rhs_j,
 // rhs = (W_v, Q^1_v, ..., Q^d_v) (eq. maxwell_def).
 template <int D, int SYS, typename T>
-__global__ void sx_relax_kernel(SxArgs S)
+__global__ void sx_relax_kernel(const __grid_constant__ SxArgs S)
 {
     constexpr int M = nvars(D, SYS);
     constexpr int NV = D + 1;
     T* f = static_cast<T*>(S.f);
-    const T omega = T(S.omega);
-    const T gm1 = T(S.gamma - 1.0);
-    T minv[NV][NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i)
-#pragma unroll
-        for (int j = 0; j < NV; ++j) minv[i][j] = T(S.minv[i * NV + j]);
+    const RelaxK<T>& RK = relax_k<T>(S.rx);
+    auto minv = [&](int i, int j) -> T {
+        if constexpr (sizeof(T) == 4) return S.minvf[i * NV + j];
+        else return S.minv[i * NV + j];
+    };
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.nodes;
          i += (long long)gridDim.x * blockDim.x) {
         T fk[NV * M];
@@ -802,13 +800,13 @@ __global__ void sx_relax_kernel(SxArgs S)
         T Q[D][M];
         if (SYS == kAdvection) {
 #pragma unroll
-            for (int a = 0; a < D; ++a) Q[a][0] = T(S.adv[a]) * W[0];
+            for (int a = 0; a < D; ++a) Q[a][0] = RK.adv[a] * W[0];
         } else {
             const T inv = T(1) / W[0];
             T ke = 0;
 #pragma unroll
             for (int b = 0; b < D; ++b) ke = fma(W[1 + b], W[1 + b], ke);
-            const T pr = gm1 * (W[1 + D] - T(0.5) * ke * inv);
+            const T pr = RK.gm1 * (W[1 + D] - T(0.5) * ke * inv);
 #pragma unroll
             for (int a = 0; a < D; ++a) {
                 const T ua = W[1 + a] * inv;
@@ -822,11 +820,11 @@ __global__ void sx_relax_kernel(SxArgs S)
         for (int kk = 0; kk < NV; ++kk)
 #pragma unroll
             for (int v = 0; v < M; ++v) {
-                T mk = minv[kk][0] * W[v];
+                T mk = minv(kk, 0) * W[v];
 #pragma unroll
-                for (int a = 0; a < D; ++a) mk = fma(minv[kk][1 + a], Q[a][v], mk);
+                for (int a = 0; a < D; ++a) mk = fma(minv(kk, 1 + a), Q[a][v], mk);
                 T& fv = fk[kk * M + v];
-                fv = (S.omega == 2.0) ? fma(T(2), mk, -fv) : omega * mk + (T(1) - omega) * fv;
+                fv = S.rx.two ? fma(T(2), mk, -fv) : RK.omega * mk + RK.om1 * fv;
             }
 #pragma unroll
         for (int p = 0; p < NV * M; ++p) f[(long long)p * S.nodes + i] = fk[p];

@@ -582,7 +582,7 @@ template <int SYS, typename V>
 __device__ __forceinline__ void tet_flux(const TetArgs& A, const V* W, int a, V* Q)
 {
     if constexpr (SYS == kAdvection) {
-        Q[0] = V(A.adv[a]) * W[0];
+        Q[0] = relax_k<V>(A.rx).adv[a] * W[0];
     } else if constexpr (SYS == kMaxwell) {
         maxwell_flux(W, a, Q, V(0));
     } else {
@@ -590,7 +590,7 @@ __device__ __forceinline__ void tet_flux(const TetArgs& A, const V* W, int a, V*
 #pragma unroll
         for (int b = 0; b < 3; ++b) ke = fma(W[1 + b], W[1 + b], ke);
         const V inv = V(1) / W[0];
-        const V pr = V(A.gamma - 1.0) * (W[4] - V(0.5) * ke * inv);
+        const V pr = relax_k<V>(A.rx).gm1 * (W[4] - V(0.5) * ke * inv);
         const V ua = W[1 + a] * inv;
         Q[0] = W[1 + a];
 #pragma unroll
@@ -611,7 +611,7 @@ __device__ __forceinline__ void tet_equilibria(const TetArgs& A, const V* W, V* 
     for (int a = 0; a < 3; ++a) tet_flux<SYS>(A, W, a, Q[a]);
     if constexpr (VS == 1) {
         constexpr int sg[4][3] = {{1, 1, 1}, {1, -1, -1}, {-1, 1, -1}, {-1, -1, 1}};
-        const V il = V(1.0 / (4.0 * A.lambda));
+        const V il = relax_k<V>(A.rx).inv4l;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -622,7 +622,7 @@ __device__ __forceinline__ void tet_equilibria(const TetArgs& A, const V* W, V* 
                 M[k * m + v] = fma(q, il, W[v] * V(0.25));
             }
     } else {
-        const V il = V(1.0 / (2.0 * A.lambda));
+        const V il = relax_k<V>(A.rx).inv2l;
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -640,7 +640,7 @@ __device__ __forceinline__ void tet_equilibria(const TetArgs& A, const V* W, V* 
 // f <- M(W+) + (1 - omega)(f - M(W-)).  Compiled per system and velocity
 // set, so that every population stays in registers.
 template <int SYS, int VS, bool EXTRAP, typename T>
-__global__ void __launch_bounds__(256) tet_relax_kernel(TetArgs A, const T* __restrict__ star)
+__global__ void __launch_bounds__(256) tet_relax_kernel(const __grid_constant__ TetArgs A, const T* __restrict__ star)
 {
     constexpr int m = nvars(3, SYS), NV = VS == 1 ? 4 : 6, NPOP = NV * m;
     T* f = static_cast<T*>(A.f);
@@ -663,21 +663,21 @@ __global__ void __launch_bounds__(256) tet_relax_kernel(TetArgs A, const T* __re
         }
         T Mm[NPOP];
         tet_equilibria<SYS, VS>(A, W, Mm);
-        const T om = T(A.omega);
+        const T om = relax_k<T>(A.rx).omega, om1 = relax_k<T>(A.rx).om1;
         if constexpr (SYS == kMaxwell) {
             T Wp[m], Mp[NPOP];
 #pragma unroll
-            for (int v = 0; v < m; ++v) Wp[v] = v < 3 ? T(A.mu) * W[v] : W[v];
+            for (int v = 0; v < m; ++v) Wp[v] = v < 3 ? relax_k<T>(A.rx).mu * W[v] : W[v];
             tet_equilibria<SYS, VS>(A, Wp, Mp);
 #pragma unroll
-            for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = fma(T(1) - om, fk[p] - Mm[p], Mp[p]);
+            for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = fma(om1, fk[p] - Mm[p], Mp[p]);
         } else {
-            if (A.omega == 2.0) {
+            if (A.rx.two) {
 #pragma unroll
                 for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = fma(T(2), Mm[p], -fk[p]);
             } else {
 #pragma unroll
-                for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = om * Mm[p] + (T(1) - om) * fk[p];
+                for (int p = 0; p < NPOP; ++p) f[p * nodes + i] = om * Mm[p] + om1 * fk[p];
             }
         }
     }
