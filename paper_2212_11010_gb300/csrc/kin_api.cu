@@ -61,6 +61,9 @@ struct kin_ctx {
     int smem = 0, grid = 0, stages = 1, threads = kThreads;
     int want_threads = 0, want_stages = 0;
     bool fixed = false;                    // compile-time block shape kernel in use
+    const void* multi = nullptr;           // several steps per launch (1D, kin_step_d1.cu)
+    size_t multi_smem = 0;
+    int multi_blocks = 1;
     // d + 1 velocity sets
     bool simplex = false;
     int vsgn[4][3] = {};
@@ -452,7 +455,17 @@ static cudaError_t configure_launch(kin_ctx* c)
     if (occ < 1) occ = 1;
     const long long ntiles = (long long)c->nblk[0] * c->nblk[1] * c->nblk[2];
     c->grid = (int)std::min<long long>(ntiles, (long long)occ * nsm);
-    return cudaSuccess;
+    c->multi = nullptr;
+    if (c->dim == 1 && c->want_stages == 0 && c->want_threads == 0 && c->debug_flags == 0) {
+        const MultiKernel mk = multi_kernel_d1(c->degree, c->system, c->precision, c->n[0], c->B[0]);
+        if (mk.fn) {
+            e = cudaFuncSetAttribute(mk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mk.smem);
+            c->multi = mk.fn;
+            c->multi_smem = mk.smem;
+            c->multi_blocks = mk.blocks;
+        }
+    }
+    return e;
 }
 
 // Launch of the fused kernel: mode 0 = one full step (reads the summaries
@@ -472,6 +485,30 @@ static kin_status launch_step_on(kin_ctx* c, int mode, cudaStream_t st)
                                  (size_t)c->smem, st));
     if (mode == 0) c->cur ^= 1;
     return KIN_OK;
+}
+
+// nsteps steps in one launch (1D problems small enough for one cluster): the
+// summaries end up in the buffer that nsteps single steps would leave them in.
+static cudaError_t launch_multi(const kin_ctx* c, const Inst& I0, int nsteps, cudaStream_t st)
+{
+    Inst I = I0;
+    if (nsteps % 2 == 0) {
+        I.sig_out = const_cast<void*>(I.sig_in);
+        I.raw_out = const_cast<void*>(I.raw_in);
+    }
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = c->multi_blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c->multi_blocks);
+    cfg.blockDim = dim3(kMultiThreads);
+    cfg.dynamicSmemBytes = c->multi_smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    void* args[] = {&I, &nsteps};
+    return cudaLaunchKernelExC(&cfg, c->multi, args);
 }
 
 static kin_status launch_step(kin_ctx* c, int mode) { return launch_step_on(c, mode, c->stream); }
@@ -1511,6 +1548,12 @@ kin_status kin_step(kin_ctx* c, int nsteps)
         if (st) return st;
         c->sum_stale = false;
     }
+    if (c->multi && nsteps > 0) {
+        KIN_CUDA(c, launch_multi(c, make_inst(c, 0), nsteps, c->stream));
+        c->cur ^= nsteps & 1;
+        c->steps_done += nsteps;
+        return KIN_OK;
+    }
     for (int s = 0; s < nsteps; ++s) {
         st = c->tet ? tet_step(c) : (c->simplex ? sx_step(c) : launch_step(c, 0));
         if (st) return st;
@@ -1781,6 +1824,7 @@ static cudaError_t batch_launch(kin_batch* b, size_t k, int q, cudaStream_t st, 
         I.raw_out = c->raw[c->cur];
     }
     c->cur = saved;
+    if (c->multi && !prep) return launch_multi(c, I, 1, st);      // bitwise what kin_step does
     void* args[] = {&I};
     return cudaLaunchKernel((const void*)c->kfn, dim3(c->grid), dim3(c->threads), args, (size_t)c->smem, st);
 }

@@ -235,6 +235,16 @@ int fixed_default_stages(int dim, int degree, int system, int prec, const int B[
 // returns the count written (at most 4).
 int fixed_shapes(int dim, int degree, int system, int prec, int out[4][3]);
 
+// 1D problems that run all steps of a call in one launch of one thread-block
+// cluster: fn(Inst, int nsteps); fn == nullptr when the problem is too large.
+constexpr int kMultiThreads = 512;
+struct MultiKernel {
+    const void* fn;
+    size_t smem;
+    int blocks;              // blocks of the cluster
+};
+MultiKernel multi_kernel_d1(int degree, int system, int prec, int n, int B);
+
 // Step kernels, one translation unit per space dimension.
 StepKernel step_kernel_d1(int degree, int system, int prec);
 StepKernel step_kernel_d2(int degree, int system, int prec);
