@@ -117,6 +117,7 @@ cudaError_t sx_launch_trace0(const SxArgs& a, int prec, cudaStream_t st);
 // velocity (split) or one for all.
 struct SxPlan {
     int threads, bpv, split, occupancy;
+    int brick;           // 2 x 2 x 2 cells per lane and wave (3D, p = 1, FP32)
     size_t smem;
 };
 int sx_sweep_shape(const SxArgs& a, int prec, SxPlan* plan);   // host only: 0 if no shape fits

@@ -771,6 +771,282 @@ __global__ void __launch_bounds__(MAXT) sx_wave_kernel(const __grid_constant__ S
     else if (D == 3) sx_sweep_velocity<D, P, 3, T>(A, lb, xs, ring);
 }
 
+// ---------------------------------------------------------------------------
+// brick sweep: 3D, p = 1, FP32
+// ---------------------------------------------------------------------------
+
+// With one cell per lane and wave, four fifths of a warp's instructions were
+// bookkeeping: positions, inflow selection, boundary lanes' branches (455 warp
+// instructions per wave of 84 FMAs, 21 of 32 lanes active).  Here a lane takes a
+// brick of 2 x 2 x 2 cells per wave, so that the bookkeeping is shared by
+// eight solves, and a warp is a unit of its own: 32 / cols streams of
+// problems, cols = (L0 / 2)(L1 / 2) lanes each, the brick columns of a
+// subdomain along z.  The schedule is sx_sweep_velocity's on bricks: lane
+// (ox, oy) runs ox + oy waves behind, so its upwind neighbours' outflow faces
+// of the wave before are the ones it needs, and they come by shuffle; along z
+// they are its own.  Nothing is shared between warps: no block barrier.
+//   The cells' f^n arrive one wave ahead by cp.async, copied by the whole warp
+// (16 lanes per brick, so that every 32-byte sector is used), the interface
+// inflow of boundary lanes beside them.  The last iterate's f^{n+1} goes back
+// the same way.  The cell solve is the one of sx_sweep_velocity, operation by
+// operation: the results are bitwise the same.
+//   Measured, D3Q4 128^3 cells, 8^3-cell subdomains: 201 us per launch (one
+// velocity, one iterate) before, 155 now, 2.85 -> 2.29 ms per step.  Nine warps
+// fit per SM (25 KB of slots and 138 registers each), so what bounds it now is
+// their latency, not the instructions.
+constexpr int kBrU = 68;              // shared-memory floats per lane: 64 values, an odd number of 16-byte words
+constexpr int kBrF = 20;              // floats per interface face: 16 values, likewise
+
+struct BrickShape {
+    int bx, by, cols, nst;            // brick columns per axis, lanes per stream, streams per warp
+    size_t smem;
+};
+
+__host__ __device__ inline BrickShape brick_shape(int L0, int L1)
+{
+    BrickShape b;
+    b.bx = L0 / 2;
+    b.by = L1 / 2;
+    b.cols = b.bx * b.by;
+    b.nst = b.cols > 0 && b.cols <= 32 ? 32 / b.cols : 0;
+    b.smem = 2 * sizeof(float) * (size_t)(32 * kBrU + (32 + b.nst * (b.bx + b.by)) * kBrF);
+    return b;
+}
+
+template <int KV>
+__device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, const int lb, float* sm)
+{
+    constexpr int SG[3] = {sx_sign(3, KV, 0), sx_sign(3, KV, 1), sx_sign(3, KV, 2)};
+    constexpr bool R0 = SG[0] > 0 || SG[1] > 0 || SG[2] > 0;
+    const SxArgs& S = A.S;
+    const BrickShape bs = brick_shape(S.L[0], S.L[1]);
+    const int lane = threadIdx.x;
+    const int str = lane / bs.cols, col = lane - str * bs.cols;
+    const int oy = col / bs.bx, ox = col - oy * bs.bx;
+    const bool active = str < bs.nst;
+    const int bz = S.L[2] / 2, skew = ox + oy, maxskew = bs.bx + bs.by - 2;
+    const int nsub = S.NS[0] * S.NS[1] * S.NS[2], nprob = S.m * nsub;
+    const int nstreams = A.bpv * bs.nst, sid = lb * bs.nst + str;
+    // problems of this stream; the warp runs as long as its first stream, which has the most
+    const int mine = active && sid < nprob ? (nprob - sid + nstreams - 1) / nstreams : 0;
+    const int most = lb * bs.nst < nprob ? (nprob - lb * bs.nst + nstreams - 1) / nstreams : 0;
+    const int span = mine * bz, total = most > 0 ? most * bz + maxskew : 0;
+    float* const f = static_cast<float*>(S.f);
+    const int n0 = S.n[0], n01 = S.n[0] * S.n[1];
+
+    const int slotf = 32 * kBrU + (32 + bs.nst * (bs.bx + bs.by)) * kBrF;
+    auto u_of = [&](int sl, int ln) { return sm + sl * slotf + ln * kBrU; };
+    auto z_of = [&](int sl) { return sm + sl * slotf + 32 * kBrU + lane * kBrF; };
+    auto x_of = [&](int sl) { return sm + sl * slotf + 32 * (kBrU + kBrF) + (str * bs.by + oy) * kBrF; };
+    auto y_of = [&](int sl) {
+        return sm + sl * slotf + 32 * (kBrU + kBrF) + (bs.nst * bs.by + str * bs.bx + ox) * kBrF;
+    };
+
+    // this lane's position: its brick's first cell, variable and subdomain
+    struct Pos {
+        int q, od, i, pop, s[3], g[3];
+        bool valid;
+    };
+    auto advance = [&](Pos& t) {
+        ++t.q;
+        t.valid = t.q >= 0 && t.q < span;
+        if (!t.valid) return;
+        if (t.q == 0 || ++t.od == bz) {
+            t.od = 0;
+            if (t.q != 0) ++t.i;
+            const int pid = sid + t.i * nstreams;
+            const int v = sx_div(pid, A.div_nsub), s = pid - v * nsub;
+            const int s12 = sx_div(s, A.div_ns0), s2 = sx_div(s12, A.div_ns1);
+            t.pop = KV * S.m + v;
+            t.s[0] = s - s12 * S.NS[0];
+            t.s[1] = s12 - s2 * S.NS[1];
+            t.s[2] = s2;
+            t.g[0] = t.s[0] * S.L[0] + (SG[0] > 0 ? 2 * ox : S.L[0] - 2 - 2 * ox);
+            t.g[1] = t.s[1] * S.L[1] + (SG[1] > 0 ? 2 * oy : S.L[1] - 2 - 2 * oy);
+        }
+        t.g[2] = t.s[2] * S.L[2] + (SG[2] > 0 ? 2 * t.od : S.L[2] - 2 - 2 * t.od);
+    };
+    auto offset = [&](const Pos& t) {
+        return t.valid ? (long long)t.pop * S.nodes + (long long)(t.g[2] * n01 + t.g[1] * n0 + t.g[0]) * 8 : -1LL;
+    };
+    auto upper = [](long long v) { return (int)(v >> 32); };
+    // the warp's bricks, 16 lanes each: lane c of 16 moves word c (row c / 4: y, then z)
+    const int cq = lane & 15, crow = (cq & 3) * 4 + ((cq >> 2) & 1) * n0 * 8 + (cq >> 3) * n01 * 8;
+    auto word_src = [&](long long off, int r, int& owner) -> long long {
+        owner = 2 * r + (lane >> 4);
+        const int lo = __shfl_sync(0xffffffffu, (int)off, owner), hi = __shfl_sync(0xffffffffu, upper(off), owner);
+        return ((long long)hi << 32) | (unsigned)lo;
+    };
+
+    // interface inflow of one axis (2 x 2 cells, 4 values each), oriented order of the transverse cells
+    auto inflow = [&](const Pos& t, int a, float* dst) {
+        const int sg = SG[a], b1 = a == 0 ? 1 : 0, b2 = a == 2 ? 1 : 2;
+#pragma unroll
+        for (int c2 = 0; c2 < 2; ++c2)
+#pragma unroll
+            for (int c1 = 0; c1 < 2; ++c1) {
+                const int g1 = t.g[b1] + (SG[b1] > 0 ? c1 : 1 - c1), g2 = t.g[b2] + (SG[b2] > 0 ? c2 : 1 - c2);
+                float* const d = dst + (2 * c2 + c1) * 4;
+                if (S.from_f) {
+                    int g[3];
+                    g[b1] = g1;
+                    g[b2] = g2;
+                    g[a] = t.g[a] + (sg > 0 ? -1 : 2);
+                    if (g[a] < 0) g[a] += S.n[a];
+                    if (g[a] >= S.n[a]) g[a] -= S.n[a];
+                    const float* up = f + (long long)t.pop * S.nodes + (long long)(g[2] * n01 + g[1] * n0 + g[0]) * 8;
+#pragma unroll
+                    for (int tt = 0; tt < 4; ++tt) cp_small_g2s<4>(d + tt, up + sx_node<3, 2>(a, sg > 0 ? 1 : 0, tt));
+                } else {
+                    int sup = t.s[a] - sg;
+                    if (sup < 0) sup += S.NS[a];
+                    if (sup >= S.NS[a]) sup -= S.NS[a];
+                    cp16_g2s(d, static_cast<const float*>(S.tr_in[a]) + ((long long)t.pop * S.NS[a] + sup) * S.glines[a] +
+                                    (long long)(g2 * S.n[b1] + g1) * 4);
+                }
+            }
+    };
+    auto fetch = [&](const Pos& t, int sl) {
+        const long long off = offset(t);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            int owner;
+            const long long o = word_src(off, r, owner);
+            if (o >= 0) cp16_g2s(u_of(sl, owner) + cq * 4, f + o + crow);
+        }
+        if (t.valid) {
+            if (ox == 0) inflow(t, 0, x_of(sl));
+            if (oy == 0) inflow(t, 1, y_of(sl));
+            if (t.od == 0) inflow(t, 2, z_of(sl));
+        }
+        cp_commit();
+    };
+    // outflow faces of a brick on the subdomain's downwind boundary
+    auto trace = [&](const Pos& t, int a, const float (&w)[2][2][4]) {
+        const int b1 = a == 0 ? 1 : 0, b2 = a == 2 ? 1 : 2;
+        float* tr = static_cast<float*>(S.tr_out[a]) + ((long long)t.pop * S.NS[a] + t.s[a]) * S.glines[a];
+#pragma unroll
+        for (int c2 = 0; c2 < 2; ++c2)
+#pragma unroll
+            for (int c1 = 0; c1 < 2; ++c1) {
+                const int g1 = t.g[b1] + (SG[b1] > 0 ? c1 : 1 - c1), g2 = t.g[b2] + (SG[b2] > 0 ? c2 : 1 - c2);
+                sx_st<4>(tr + (long long)(g2 * S.n[b1] + g1) * 4, w[c2][c1]);
+            }
+    };
+
+    // faces [c2][c1][4], the transverse cells in oriented order: inflow before
+    // a cell's solve, its outflow after it
+    float fx[2][2][4] = {}, fy[2][2][4] = {}, fz[2][2][4] = {};
+    Pos tp, tc;
+    tp.q = -skew - 1;
+    tp.od = tp.i = tp.pop = 0;
+    tp.valid = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) tp.s[a] = tp.g[a] = 0;
+    advance(tp);
+    fetch(tp, 0);
+    for (int W = 0; W < total; ++W) {
+        const int sl = W & 1;
+        tc = tp;
+        advance(tp);
+        fetch(tp, sl ^ 1);
+        cp_wait_group<1>();
+        __syncwarp();                 // this wave's copies, by every lane, have landed
+        // transverse inflow: the neighbour's faces of the wave before
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            float* px = &fx[0][0][0] + c;
+            float* py = &fy[0][0][0] + c;
+            *px = __shfl_up_sync(0xffffffffu, *px, 1);
+            *py = __shfl_up_sync(0xffffffffu, *py, bs.bx);
+        }
+        if (tc.valid) {
+            auto take = [&](const float* p, float (&w)[2][2][4]) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) sx_lds<4, true>(p + 4 * c, &w[0][0][0] + 4 * c);
+            };
+            if (ox == 0) take(x_of(sl), fx);
+            if (oy == 0) take(y_of(sl), fy);
+            if (tc.od == 0) take(z_of(sl), fz);
+            float* const ub = u_of(sl, lane);
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        float* const uc = ub + (SG[2] > 0 ? k : 1 - k) * 32 + (SG[1] > 0 ? j : 1 - j) * 16 +
+                                          (SG[0] > 0 ? i : 1 - i) * 8;
+                        float u[8], r[8], x[8];
+                        sx_lds<8, true>(uc, u);
+                        const float tref = u[0];
+                        r[0] = 0.0f;
+#pragma unroll
+                        for (int n = 1; n < 8; ++n) r[n] = A.wcell[n] * (u[n] - tref);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            const float* tv = a == 0 ? fx[k][j] : (a == 1 ? fy[k][i] : fz[j][i]);
+#pragma unroll
+                            for (int tt = 0; tt < 4; ++tt) {
+                                const int n = sx_node<3, 2>(a, SG[a] > 0 ? 0 : 1, tt);
+                                r[n] = fmaf(A.face[KV][a][tt], tv[tt] - tref, r[n]);
+                            }
+                        }
+#pragma unroll
+                        for (int n = 0; n < 8; ++n)
+                            x[n] = R0 ? A.ainv[KV][n * 8] * r[0] : A.ainv[KV][n * 8 + 1] * r[1];
+#pragma unroll
+                        for (int c = R0 ? 1 : 2; c < 8; ++c)
+#pragma unroll
+                            for (int n = 0; n < 8; ++n) x[n] = fmaf(A.ainv[KV][n * 8 + c], r[c], x[n]);
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) x[n] += tref;
+#pragma unroll
+                        for (int tt = 0; tt < 4; ++tt) {
+                            fx[k][j][tt] = x[sx_node<3, 2>(0, SG[0] > 0 ? 1 : 0, tt)];
+                            fy[k][i][tt] = x[sx_node<3, 2>(1, SG[1] > 0 ? 1 : 0, tt)];
+                            fz[j][i][tt] = x[sx_node<3, 2>(2, SG[2] > 0 ? 1 : 0, tt)];
+                        }
+                        if (S.final_iter) {
+#pragma unroll
+                            for (int n = 0; n < 8; ++n) x[n] = fmaf(2.0f, x[n], -u[n]);
+                            sx_sts<8, true>(uc, x);
+                        }
+                    }
+            if (!S.final_iter) {
+                if (ox == bs.bx - 1) trace(tc, 0, fx);
+                if (oy == bs.by - 1) trace(tc, 1, fy);
+                if (tc.od == bz - 1) trace(tc, 2, fz);
+            }
+        }
+        __syncwarp();                 // the slot may be refilled; the last iterate's values are in it
+        if (S.final_iter) {
+            const long long off = offset(tc);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                int owner;
+                const long long o = word_src(off, r, owner);
+                if (o >= 0)
+                    *reinterpret_cast<float4*>(f + o + crow) = *reinterpret_cast<const float4*>(u_of(sl, owner) + cq * 4);
+            }
+            __syncwarp();
+        }
+    }
+    cp_wait_group<0>();
+}
+
+// One warp per block: blockIdx.x / bpv + k0 is the velocity.
+__global__ void __launch_bounds__(32) sx_brick_kernel(const __grid_constant__ SxWave<3, 1, float> A)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float* sm = reinterpret_cast<float*>(smem_raw);
+    const int k = A.k0 + (int)blockIdx.x / A.bpv, lb = (int)blockIdx.x % A.bpv;
+    if (k == 0) sx_brick_velocity<0>(A, lb, sm);
+    else if (k == 1) sx_brick_velocity<1>(A, lb, sm);
+    else if (k == 2) sx_brick_velocity<2>(A, lb, sm);
+    else sx_brick_velocity<3>(A, lb, sm);
+}
+
 // Relaxation with the d + 1 velocity equilibria: M_{k,v} = sum_j Minv[k][j] rhs_j,
 // rhs = (W_v, Q^1_v, ..., Q^d_v) (eq. maxwell_def).
 template <int D, int SYS, typename T>
@@ -961,9 +1237,21 @@ int sx_sweep_shape(const SxArgs& a, int prec, SxPlan* plan)
 cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
 {
     if (!sx_sweep_shape(a, prec, plan)) return cudaErrorInvalidValue;
-    const void* fn = prec == 1 ? wave_pick<float>(a.dim, a.degree, plan->threads)
-                               : wave_pick<double>(a.dim, a.degree, plan->threads);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem);
+    // subdomains of whole 2 x 2 x 2 bricks with at most a warp of brick columns
+    const bool even = a.dim == 3 && a.degree == 1 && a.L[0] % 2 == 0 && a.L[1] % 2 == 0 && a.L[2] % 2 == 0;
+    const BrickShape bs = brick_shape(a.L[0], a.L[1]);
+    plan->brick = prec == 1 && even && bs.nst > 0;
+    if (plan->brick) {
+        plan->threads = 32;
+        plan->smem = bs.smem;
+    }
+    const void* fn = (const void*)sx_brick_kernel;
+    if (!plan->brick)
+        fn = prec == 1 ? wave_pick<float>(a.dim, a.degree, plan->threads)
+                       : wave_pick<double>(a.dim, a.degree, plan->threads);
+    // (the brick kernel's shared memory stays below 48 KB)
+    cudaError_t e = plan->brick ? cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)
+                                : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem);
     if (e != cudaSuccess) return e;
     int occ = 0, dev = 0, nsm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, plan->threads, plan->smem);
@@ -975,7 +1263,8 @@ cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
     // problems.  When one velocity's problems alone fill that wave, the
     // velocities go in separate launches (an SM then runs one velocity's
     // code at a time); otherwise one launch takes them all.
-    const int nprob = a.m * a.NS[0] * a.NS[1] * a.NS[2];
+    const int nst = plan->brick ? bs.nst : 1;                  // problem streams per block
+    const int nprob = (a.m * a.NS[0] * a.NS[1] * a.NS[2] + nst - 1) / nst;
     const int slots = occ * nsm;
     plan->split = nprob >= slots;
     int b = plan->split ? slots : slots / a.nvel;
@@ -1010,6 +1299,8 @@ static cudaError_t wave_launch(const SxArgs& a, const double* hrec, int rstride,
     }
     for (int j = 0; j < NN; ++j) w.wcell[j] = (T)hrec[NN * NN + j];
     const void* fn = wave_fn<D, P, T>(plan.threads);
+    if constexpr (D == 3 && P == 1 && sizeof(T) == 4)
+        if (plan.brick) fn = (const void*)sx_brick_kernel;
     void* p[] = {&w};
     if (!plan.split)
         return cudaLaunchKernel(fn, dim3(a.nvel * plan.bpv), dim3(plan.threads), p, plan.smem, st);
