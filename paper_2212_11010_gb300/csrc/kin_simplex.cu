@@ -785,15 +785,18 @@ __global__ void __launch_bounds__(MAXT) sx_wave_kernel(const __grid_constant__ S
 // (ox, oy) runs ox + oy waves behind, so its upwind neighbours' outflow faces
 // of the wave before are the ones it needs, and they come by shuffle; along z
 // they are its own.  Nothing is shared between warps: no block barrier.
-//   The cells' f^n arrive one wave ahead by cp.async, copied by the whole warp
-// (16 lanes per brick, so that every 32-byte sector is used), the interface
-// inflow of boundary lanes beside them.  The last iterate's f^{n+1} goes back
-// the same way.  The cell solve is the one of sx_sweep_velocity, operation by
+//   The cells' f^n arrive by cp.async, copied by the whole warp (8 lanes per half
+// brick, so that every 32-byte sector is used): once the four cells of a half
+// are solved, the next brick's half takes their place while the other half is
+// solved, so one brick of shared memory per lane is enough.  The interface
+// inflow of boundary lanes comes beside them, and the last iterate's f^{n+1}
+// goes back the same way.  The cell solve is the one of sx_sweep_velocity, operation by
 // operation: the results are bitwise the same.
 //   Measured, D3Q4 128^3 cells, 8^3-cell subdomains: 201 us per launch (one
-// velocity, one iterate) before, 155 now, 2.85 -> 2.29 ms per step.  Nine warps
-// fit per SM (25 KB of slots and 138 registers each), so what bounds it now is
-// their latency, not the instructions.
+// velocity, one iterate) before, 146 now, 2.85 -> 2.17 ms per step.  Twelve warps
+// fit per SM (137 registers); with two bricks per lane it was eight and 155 us,
+// with the registers cut to 128 for sixteen 153 us.  1,550 warp instructions per
+// wave, 920 of them the solves, are issued at 45% of the rate.
 constexpr int kBrU = 68;              // shared-memory floats per lane: 64 values, an odd number of 16-byte words
 constexpr int kBrF = 20;              // floats per interface face: 16 values, likewise
 
@@ -809,7 +812,7 @@ __host__ __device__ inline BrickShape brick_shape(int L0, int L1)
     b.by = L1 / 2;
     b.cols = b.bx * b.by;
     b.nst = b.cols > 0 && b.cols <= 32 ? 32 / b.cols : 0;
-    b.smem = 2 * sizeof(float) * (size_t)(32 * kBrU + (32 + b.nst * (b.bx + b.by)) * kBrF);
+    b.smem = sizeof(float) * (size_t)(32 * kBrU + (32 + b.nst * (b.bx + b.by)) * kBrF);
     return b;
 }
 
@@ -834,13 +837,9 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
     float* const f = static_cast<float*>(S.f);
     const int n0 = S.n[0], n01 = S.n[0] * S.n[1];
 
-    const int slotf = 32 * kBrU + (32 + bs.nst * (bs.bx + bs.by)) * kBrF;
-    auto u_of = [&](int sl, int ln) { return sm + sl * slotf + ln * kBrU; };
-    auto z_of = [&](int sl) { return sm + sl * slotf + 32 * kBrU + lane * kBrF; };
-    auto x_of = [&](int sl) { return sm + sl * slotf + 32 * (kBrU + kBrF) + (str * bs.by + oy) * kBrF; };
-    auto y_of = [&](int sl) {
-        return sm + sl * slotf + 32 * (kBrU + kBrF) + (bs.nst * bs.by + str * bs.bx + ox) * kBrF;
-    };
+    float* const zin = sm + 32 * kBrU + lane * kBrF;
+    float* const xin = sm + 32 * (kBrU + kBrF) + (str * bs.by + oy) * kBrF;
+    float* const yin = sm + 32 * (kBrU + kBrF) + (bs.nst * bs.by + str * bs.bx + ox) * kBrF;
 
     // this lane's position: its brick's first cell, variable and subdomain
     struct Pos {
@@ -870,12 +869,18 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
         return t.valid ? (long long)t.pop * S.nodes + (long long)(t.g[2] * n01 + t.g[1] * n0 + t.g[0]) * 8 : -1LL;
     };
     auto upper = [](long long v) { return (int)(v >> 32); };
-    // the warp's bricks, 16 lanes each: lane c of 16 moves word c (row c / 4: y, then z)
-    const int cq = lane & 15, crow = (cq & 3) * 4 + ((cq >> 2) & 1) * n0 * 8 + (cq >> 3) * n01 * 8;
-    auto word_src = [&](long long off, int r, int& owner) -> long long {
-        owner = 2 * r + (lane >> 4);
-        const int lo = __shfl_sync(0xffffffffu, (int)off, owner), hi = __shfl_sync(0xffffffffu, upper(off), owner);
-        return ((long long)hi << 32) | (unsigned)lo;
+    // the warp's half bricks (two cells along z: oriented half h), 8 lanes
+    // each: lane c of 8 moves word c & 3 of row c / 4
+    const int cq = lane & 7, cword = (cq & 3) * 4, crow = cq >> 2;
+    auto each_word = [&](long long off, int h, auto&& go) {
+        const int z = SG[2] > 0 ? h : 1 - h, src = cword + crow * n0 * 8 + z * n01 * 8;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int owner = 4 * r + (lane >> 3);
+            const int lo = __shfl_sync(0xffffffffu, (int)off, owner), hi = __shfl_sync(0xffffffffu, upper(off), owner);
+            const long long o = ((long long)hi << 32) | (unsigned)lo;
+            if (o >= 0) go(f + o + src, sm + owner * kBrU + z * 32 + crow * 16 + cword);
+        }
     };
 
     // interface inflow of one axis (2 x 2 cells, 4 values each), oriented order of the transverse cells
@@ -906,18 +911,12 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
                 }
             }
     };
-    auto fetch = [&](const Pos& t, int sl) {
-        const long long off = offset(t);
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            int owner;
-            const long long o = word_src(off, r, owner);
-            if (o >= 0) cp16_g2s(u_of(sl, owner) + cq * 4, f + o + crow);
-        }
-        if (t.valid) {
-            if (ox == 0) inflow(t, 0, x_of(sl));
-            if (oy == 0) inflow(t, 1, y_of(sl));
-            if (t.od == 0) inflow(t, 2, z_of(sl));
+    auto fetch = [&](const Pos& t, int h) {
+        each_word(offset(t), h, [](float* g, float* d) { cp16_g2s(d, g); });
+        if (h == 0 && t.valid) {
+            if (ox == 0) inflow(t, 0, xin);
+            if (oy == 0) inflow(t, 1, yin);
+            if (t.od == 0) inflow(t, 2, zin);
         }
         cp_commit();
     };
@@ -945,13 +944,10 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
     for (int a = 0; a < 3; ++a) tp.s[a] = tp.g[a] = 0;
     advance(tp);
     fetch(tp, 0);
+    fetch(tp, 1);
     for (int W = 0; W < total; ++W) {
-        const int sl = W & 1;
         tc = tp;
         advance(tp);
-        fetch(tp, sl ^ 1);
-        cp_wait_group<1>();
-        __syncwarp();                 // this wave's copies, by every lane, have landed
         // transverse inflow: the neighbour's faces of the wave before
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
@@ -960,23 +956,26 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
             *px = __shfl_up_sync(0xffffffffu, *px, 1);
             *py = __shfl_up_sync(0xffffffffu, *py, bs.bx);
         }
-        if (tc.valid) {
-            auto take = [&](const float* p, float (&w)[2][2][4]) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) sx_lds<4, true>(p + 4 * c, &w[0][0][0] + 4 * c);
-            };
-            if (ox == 0) take(x_of(sl), fx);
-            if (oy == 0) take(y_of(sl), fy);
-            if (tc.od == 0) take(z_of(sl), fz);
-            float* const ub = u_of(sl, lane);
+        for (int k = 0; k < 2; ++k) {
+            cp_wait_group<1>();           // half k has landed; the other half may be in flight
+            __syncwarp();
+            if (tc.valid) {
+                if (k == 0) {
+                    auto take = [&](const float* p, float (&w)[2][2][4]) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
+                        for (int c = 0; c < 4; ++c) sx_lds<4, true>(p + 4 * c, &w[0][0][0] + 4 * c);
+                    };
+                    if (ox == 0) take(xin, fx);
+                    if (oy == 0) take(yin, fy);
+                    if (tc.od == 0) take(zin, fz);
+                }
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
-                        float* const uc = ub + (SG[2] > 0 ? k : 1 - k) * 32 + (SG[1] > 0 ? j : 1 - j) * 16 +
-                                          (SG[0] > 0 ? i : 1 - i) * 8;
+                        float* const uc = sm + lane * kBrU + (SG[2] > 0 ? k : 1 - k) * 32 +
+                                          (SG[1] > 0 ? j : 1 - j) * 16 + (SG[0] > 0 ? i : 1 - i) * 8;
                         float u[8], r[8], x[8];
                         sx_lds<8, true>(uc, u);
                         const float tref = u[0];
@@ -1013,23 +1012,20 @@ __device__ __forceinline__ void sx_brick_velocity(const SxWave<3, 1, float>& A, 
                             sx_sts<8, true>(uc, x);
                         }
                     }
-            if (!S.final_iter) {
-                if (ox == bs.bx - 1) trace(tc, 0, fx);
-                if (oy == bs.by - 1) trace(tc, 1, fy);
-                if (tc.od == bz - 1) trace(tc, 2, fz);
+                if (k == 1 && !S.final_iter) {
+                    if (ox == bs.bx - 1) trace(tc, 0, fx);
+                    if (oy == bs.by - 1) trace(tc, 1, fy);
+                    if (tc.od == bz - 1) trace(tc, 2, fz);
+                }
             }
-        }
-        __syncwarp();                 // the slot may be refilled; the last iterate's values are in it
-        if (S.final_iter) {
-            const long long off = offset(tc);
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                int owner;
-                const long long o = word_src(off, r, owner);
-                if (o >= 0)
-                    *reinterpret_cast<float4*>(f + o + crow) = *reinterpret_cast<const float4*>(u_of(sl, owner) + cq * 4);
+            __syncwarp();                 // half k may be refilled; the last iterate's values are in it
+            if (S.final_iter) {
+                each_word(offset(tc), k, [](float* g, float* d) {
+                    *reinterpret_cast<float4*>(g) = *reinterpret_cast<const float4*>(d);
+                });
+                __syncwarp();
             }
-            __syncwarp();
+            fetch(tp, k);
         }
     }
     cp_wait_group<0>();
@@ -1237,10 +1233,19 @@ int sx_sweep_shape(const SxArgs& a, int prec, SxPlan* plan)
 cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
 {
     if (!sx_sweep_shape(a, prec, plan)) return cudaErrorInvalidValue;
-    // subdomains of whole 2 x 2 x 2 bricks with at most a warp of brick columns
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // Bricks: subdomains of whole 2 x 2 x 2 bricks with at most a warp of brick
+    // columns, and enough of them that 16 warps per SM have work -- a brick wave
+    // is eight cells long, and with few warps its latency shows (12 steps, one
+    // cell against bricks: 22 warps per SM, 48^3 cells in 6^3 subdomains, 5.5 ms
+    // against 4.0; 7 per SM, 40 x 40 x 48 cells, 2.8 against 4.1).
     const bool even = a.dim == 3 && a.degree == 1 && a.L[0] % 2 == 0 && a.L[1] % 2 == 0 && a.L[2] % 2 == 0;
     const BrickShape bs = brick_shape(a.L[0], a.L[1]);
-    plan->brick = prec == 1 && even && bs.nst > 0;
+    const long long all = (long long)a.nvel * a.m * a.NS[0] * a.NS[1] * a.NS[2];
+    plan->brick = prec == 1 && even && bs.nst > 0 && all >= 16LL * nsm * bs.nst;
     if (plan->brick) {
         plan->threads = 32;
         plan->smem = bs.smem;
@@ -1250,13 +1255,11 @@ cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
         fn = prec == 1 ? wave_pick<float>(a.dim, a.degree, plan->threads)
                        : wave_pick<double>(a.dim, a.degree, plan->threads);
     // (the brick kernel's shared memory stays below 48 KB)
-    cudaError_t e = plan->brick ? cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)
+    e = plan->brick ? cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)
                                 : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem);
     if (e != cudaSuccess) return e;
-    int occ = 0, dev = 0, nsm = 0;
+    int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, plan->threads, plan->smem);
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     // one resident wave of blocks, each streaming ceil(problems / blocks)
