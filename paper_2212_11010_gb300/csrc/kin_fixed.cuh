@@ -138,8 +138,17 @@ struct Shape {
             if (((NROWS * (ROWLEN + 4) + pp) / 4) % 8 == 1) return pp;
         return 0;
     }
-    static constexpr int RP = G4 ? 4 : best_pad(true);
-    static constexpr int PP = G4 ? g4_pp() : best_pad(false);
+    // Degree 1 in 3D (FP32): a cell is two 16-byte words that hold the four
+    // lines of any axis through it, swept together (pm_group3).  Row pad 4
+    // puts neighbouring rows an odd number of words apart; without a slab
+    // pad three 4 x 4 x 4 Euler tiles just fit an SM (76,800 bytes each).
+    static constexpr bool G3 = D == 3 && NP == 2 && sizeof(T) == 4;
+    // Four lines of one transverse cell are consecutive in the summaries: the
+    // look-back takes them as one 16-byte word (fixed_chain4).
+    static constexpr bool C4 = TN == 4 && sizeof(T) == 4;
+    static constexpr int RP = G4 || G3 ? 4 : best_pad(true);
+    static constexpr int PP = G4 ? g4_pp() : (G3 ? 0 : best_pad(false));
+    static constexpr int tcells(int a) { return CELLS / ext(a); }          // transverse cells of axis a
     static constexpr int RSTR = rstr(RP);
     static constexpr int PSTR = pstr(RP, PP);
     static constexpr int TILE = NPOP * PSTR;                        // elements per tile buffer
@@ -412,6 +421,89 @@ __device__ __forceinline__ void pm_group4(const Inst& I, int git, int org0, int 
     }
 }
 
+// Sweep (MODE 1) or block summaries (MODE 2) of the four lines of axis A
+// through one column of cells, 3D degree 1 (Shape::G3).  Group items: (sign,
+// variable) major, transverse cell fastest.  Every cell is two 16-byte words
+// whatever the axis -- node jx + 2 jy + 4 jz -- so a cell costs two loads and two
+// stores of shared memory for its eight values, and one set of coefficients and
+// addresses serves four lines.  One line per item took 4,900 shared-memory
+// wavefronts and 18,600 warp instructions per 4 x 4 x 4 tile of Euler.
+//   Measured with the look-back of fixed_chain4 (128^3 cells, per step): Euler
+// 1.15 -> 1.07 ms, Maxwell 1.55 -> 1.43.
+template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int A, int MODE, bool BATCH>
+__device__ __forceinline__ void pm_group3(const Inst& I, int local, int org0, int org1, int org2, int bidx, float* s,
+                                          const float* tin, const float* csm)
+{
+    using S = Shape<D, P, SYS, T, B0, B1, B2>;
+    constexpr int M = S::M, TC = S::tcells(A), BA = S::ext(A), CST = S::cstep(S::RP, A);
+    constexpr int T1 = S::t1(A), T2 = S::t2(A), E1 = S::ext(T1);
+    const int sg = local / (M * TC), rem = local - sg * (M * TC);
+    const int v = rem / TC, tc = rem - (rem / TC) * TC, c1 = tc % E1, c2 = tc / E1;
+    const int dir = 2 * A + sg, pop = dir * M + v;
+    int c[3] = {0, 0, 0};
+    c[T1] = c1;
+    c[T2] = c2;
+    float* p = s + pop * S::PSTR + S::cell_off(S::RP, c[0], c[1], c[2]) + (sg == 0 ? 0 : (BA - 1) * CST);
+    const int step = sg == 0 ? CST : -CST;
+    // value of line l at node j along the axis
+    auto at = [](int l, int j) { return A == 0 ? 2 * l + j : (A == 1 ? (l & 1) + 2 * j + 4 * (l >> 1) : l + 4 * j); };
+    float t[4];
+    if (MODE == 1) {
+        const float p00 = cget<BATCH>(I, csm, dir, 0), p01 = cget<BATCH>(I, csm, dir, 1);
+        const float p10 = cget<BATCH>(I, csm, dir, 2), p11 = cget<BATCH>(I, csm, dir, 3);
+        const float4 t0 = *reinterpret_cast<const float4*>(tin + sg * S::ITEMS + S::eoff(A) + v * S::lines(A) + tc * 4);
+        t[0] = t0.x;
+        t[1] = t0.y;
+        t[2] = t0.z;
+        t[3] = t0.w;
+#pragma unroll
+        for (int cc = 0; cc < BA; ++cc, p += step) {
+            const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+            float u[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                float& u0 = u[at(l, 0)];
+                float& u1 = u[at(l, 1)];
+                // difference form, as in pm_item
+                const float d0 = u0 - t[l], d1 = u1 - t[l];
+                const float x0 = fmaf(p01, d1, p00 * d0), x1 = fmaf(p11, d1, p10 * d0);
+                t[l] = sg == 0 ? u1 + x1 : u0 + x0;
+                u0 = fmaf(2.0f, x0, u0);
+                u1 = fmaf(2.0f, x1, u1);
+            }
+            *reinterpret_cast<float4*>(p) = make_float4(u[0], u[1], u[2], u[3]);
+            *reinterpret_cast<float4*>(p + 4) = make_float4(u[4], u[5], u[6], u[7]);
+        }
+    } else {
+        const float w0 = cget<BATCH>(I, csm, dir, kOffProw), w1 = cget<BATCH>(I, csm, dir, kOffProw + 1);
+        const float rho = cget<BATCH>(I, csm, dir, kOffRho);
+        float last[4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) t[l] = 0.0f;
+#pragma unroll
+        for (int cc = 0; cc < BA; ++cc, p += step) {
+            const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+            const float u[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                t[l] = fmaf(rho, t[l], fmaf(w1, u[at(l, 1)], w0 * u[at(l, 0)]));
+                if (cc == BA - 1) last[l] = sg == 0 ? u[at(l, 1)] : u[at(l, 0)];
+            }
+        }
+        const int nbk = I.nblk[A], nbs = I.nb[A];
+        const int q = sg == 0 ? bidx : nbk - 1 - bidx;
+        const int Sd = (int)fdiv((unsigned)q, I.fd_nb[A]);
+        const long long gl = I.ax[A].glines;
+        const int o1 = T1 == 0 ? org0 : org1, o2 = T2 == 1 ? org1 : org2;
+        const long long gline = ((long long)(o2 + c2) * I.n[T1] + (o1 + c1)) * 4;
+        *reinterpret_cast<float4*>(static_cast<float*>(I.sig_out) + (long long)pop * I.sig_stride + (long long)q * gl +
+                                   gline) = make_float4(t[0], t[1], t[2], t[3]);
+        if (q - Sd * nbs == nbs - 1)
+            *reinterpret_cast<float4*>(static_cast<float*>(I.raw_out) + (long long)pop * I.raw_stride +
+                                       (long long)Sd * gl + gline) = make_float4(last[0], last[1], last[2], last[3]);
+    }
+}
+
 template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH, int MODE, bool BATCH>
 __device__ __forceinline__ void fixed_pm_all(const Inst& I, int org0, int org1, int org2, int bx, int by, int bz,
                                              T* s, const T* tin, const T* csm)
@@ -425,18 +517,28 @@ __device__ __forceinline__ void fixed_pm_all(const Inst& I, int org0, int org1, 
             if (NG % NTH != 0 && git >= NG) break;
             pm_group4<D, P, SYS, T, B0, B1, B2, MODE, BATCH>(I, git, org0, org1, bx, by, s, tin, csm);
         }
-        return;
-    }
+    } else if constexpr (S::G3) {
+        constexpr int N0 = 2 * S::M * S::tcells(0), N1 = N0 + 2 * S::M * S::tcells(1), NG = N1 + 2 * S::M * S::tcells(2);
 #pragma unroll
-    for (int k = 0; k < (S::ITEMS + NTH - 1) / NTH; ++k) {
-        const int it = threadIdx.x + k * NTH;
-        if (S::ITEMS % NTH != 0 && it >= S::ITEMS) break;
-        if (it < S::E0) {
-            pm_item<D, P, SYS, T, B0, B1, B2, 0, MODE, BATCH>(I, it, org0, org1, org2, bx, s, tin, csm);
-        } else if (D == 2 || it < S::E1) {
-            if constexpr (D > 1) pm_item<D, P, SYS, T, B0, B1, B2, 1, MODE, BATCH>(I, it - S::E0, org0, org1, org2, by, s, tin, csm);
-        } else {
-            if constexpr (D > 2) pm_item<D, P, SYS, T, B0, B1, B2, 2, MODE, BATCH>(I, it - S::E1, org0, org1, org2, bz, s, tin, csm);
+        for (int k = 0; k < (NG + NTH - 1) / NTH; ++k) {
+            const int g = threadIdx.x + k * NTH;
+            if (NG % NTH != 0 && g >= NG) break;
+            if (g < N0) pm_group3<D, P, SYS, T, B0, B1, B2, 0, MODE, BATCH>(I, g, org0, org1, org2, bx, s, tin, csm);
+            else if (g < N1) pm_group3<D, P, SYS, T, B0, B1, B2, 1, MODE, BATCH>(I, g - N0, org0, org1, org2, by, s, tin, csm);
+            else pm_group3<D, P, SYS, T, B0, B1, B2, 2, MODE, BATCH>(I, g - N1, org0, org1, org2, bz, s, tin, csm);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < (S::ITEMS + NTH - 1) / NTH; ++k) {
+            const int it = threadIdx.x + k * NTH;
+            if (S::ITEMS % NTH != 0 && it >= S::ITEMS) break;
+            if (it < S::E0) {
+                pm_item<D, P, SYS, T, B0, B1, B2, 0, MODE, BATCH>(I, it, org0, org1, org2, bx, s, tin, csm);
+            } else if (D == 2 || it < S::E1) {
+                if constexpr (D > 1) pm_item<D, P, SYS, T, B0, B1, B2, 1, MODE, BATCH>(I, it - S::E0, org0, org1, org2, by, s, tin, csm);
+            } else {
+                if constexpr (D > 2) pm_item<D, P, SYS, T, B0, B1, B2, 2, MODE, BATCH>(I, it - S::E1, org0, org1, org2, bz, s, tin, csm);
+            }
         }
     }
 }
@@ -562,6 +664,93 @@ __device__ __forceinline__ void fixed_chain(const Inst& I, int org0, int org1, i
             const int it = hid + k * HALF;
             if (k < KP[A] && it < S::M * S::lines(A)) tin[sgn * S::ITEMS + S::eoff(A) + it] = tr[A][k];
         }
+}
+
+// The look-back of fixed_chain where four consecutive lines make one 16-byte
+// word (Shape::C4): a thread folds whole words, KQ of them side by side, so a
+// summary block costs one load and one address step for four lines.  (Scalar
+// lines: 70 instructions a line, a quarter of a 3D tile's.)
+template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH>
+__device__ __forceinline__ void fixed_chain4(const Inst& I, int org0, int org1, int org2, int bx, int by, int bz,
+                                             float* tin)
+{
+    using S = Shape<D, P, SYS, T, B0, B1, B2>;
+    constexpr int M = S::M;
+    constexpr int G0 = M * S::tcells(0), G1 = G0 + (D > 1 ? M * S::tcells(1) : 0), GT = G1 + (D > 2 ? M * S::tcells(2) : 0);
+    constexpr int KQ = (2 * GT + NTH - 1) / NTH;
+    const float* __restrict__ sig = static_cast<const float*>(I.sig_in);
+    float4 t[KQ];
+    float RB[KQ];
+    int idx[KQ], gl[KQ], left[KQ], nbk[KQ], cnt[KQ], dst[KQ];
+    int maxcnt = 0;
+#pragma unroll
+    for (int k = 0; k < KQ; ++k) {
+        const int g = threadIdx.x + k * NTH;
+        cnt[k] = 0;
+        dst[k] = -1;
+        if ((2 * GT) % NTH != 0 && g >= 2 * GT) continue;
+        const int sgn = g / GT, rem = g - sgn * GT;
+        const int A = rem < G0 ? 0 : (D == 2 || rem < G1 ? 1 : 2);
+        const int loc = rem - (A == 0 ? 0 : (A == 1 ? G0 : G1));
+        const int TC = A == 0 ? S::tcells(0) : (A == 1 ? S::tcells(1) : S::tcells(2));
+        const int v = loc / TC, tc = loc - v * TC;
+        const int E1 = A == 0 ? B1 : B0;
+        const int c2 = D > 2 ? tc / E1 : 0, c1 = tc - c2 * E1;
+        const int o1 = A == 0 ? org1 : org0, o2 = A == 2 ? org1 : org2;
+        const int gline = ((D > 2 ? (o2 + c2) * I.n[A == 0 ? 1 : 0] : 0) + o1 + c1) * 4;
+        const int pop = (2 * A + sgn) * M + v;
+        const int bidx = A == 0 ? bx : (A == 1 ? by : bz);
+        // the walk, as in chain_setup
+        const int nbs = I.nb[A], NSa = I.NS[A], K = I.iters;
+        nbk[k] = I.nblk[A];
+        const int q = sgn == 0 ? bidx : nbk[k] - 1 - bidx;
+        const int Sd = (int)fdiv((unsigned)q, I.fd_nb[A]), r = q - Sd * nbs;
+        int s0 = Sd - K;
+        const bool from_bnd = I.inflow[A] && s0 < 0;
+        while (s0 < 0) s0 += NSa;
+        gl[k] = (int)I.ax[A].glines;
+        int n = from_bnd ? Sd * nbs + r : (K - 1) * nbs + r;
+        int qj = from_bnd ? 0 : ((s0 + 1 == NSa) ? 0 : (s0 + 1) * nbs);
+        const int depth = I.lbdepth[2 * A + sgn];
+        const bool trunc = n > depth;
+        if (trunc) {
+            qj = (qj + n - depth) % nbk[k];
+            n = depth;
+        }
+        cnt[k] = n;
+        maxcnt = n > maxcnt ? n : maxcnt;
+        RB[k] = coef_of(I, 2 * A + sgn, kOffRhoB, 0.0f);
+        left[k] = nbk[k] - qj;
+        idx[k] = (int)((long long)pop * I.sig_stride + gline + (long long)qj * gl[k]);   // fits: checked on the host
+        dst[k] = sgn * S::ITEMS + (A == 0 ? S::eoff(0) : (A == 1 ? S::eoff(1) : S::eoff(2))) + v * TC * 4 + tc * 4;
+        if (trunc) {
+            t[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        } else if (from_bnd) {
+            const float b = __ldg(static_cast<const float*>(I.bnd) + pop);
+            t[k] = make_float4(b, b, b, b);
+        } else {
+            t[k] = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(I.raw_in) + (long long)s0 * gl[k] +
+                                                         (long long)pop * I.raw_stride + gline));
+        }
+    }
+#pragma unroll 4
+    for (int j = 0; j < maxcnt; ++j) {
+#pragma unroll
+        for (int k = 0; k < KQ; ++k)
+            if (j < cnt[k]) {
+                const float4 w = __ldg(reinterpret_cast<const float4*>(sig + idx[k]));
+                t[k].x = fmaf(RB[k], t[k].x, w.x);
+                t[k].y = fmaf(RB[k], t[k].y, w.y);
+                t[k].z = fmaf(RB[k], t[k].z, w.z);
+                t[k].w = fmaf(RB[k], t[k].w, w.w);
+                const bool wrap = --left[k] == 0;
+                idx[k] += wrap ? gl[k] - nbk[k] * gl[k] : gl[k];
+                left[k] = wrap ? nbk[k] : left[k];
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < KQ; ++k)
+        if (dst[k] >= 0) *reinterpret_cast<float4*>(tin + dst[k]) = t[k];
 }
 
 template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH>
@@ -860,11 +1049,17 @@ __device__ __forceinline__ void fixed_load(const Inst& I, int t, T* s)
     fixed_copy<D, P, SYS, T, B0, B1, B2, NTH, false>(I, c.bx * B0, c.by * B1, c.bz * B2, s);
 }
 
-template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH>
+// (batched 2D degree 3 keeps the scalar lines: with the launch record in
+// global memory the words measured 1% slower on the 24-problem batch, against
+// 2% faster on a single 512^2 problem)
+template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH, bool BATCH>
 __device__ __forceinline__ void fixed_chain_tile(const Inst& I, int t, T* tin)
 {
     const TileXYZ c = tile_xyz(I, t);
-    fixed_chain<D, P, SYS, T, B0, B1, B2, NTH>(I, c.bx * B0, c.by * B1, c.bz * B2, c.bx, c.by, c.bz, tin);
+    if constexpr (Shape<D, P, SYS, T, B0, B1, B2>::C4 && (D == 3 || !BATCH))
+        fixed_chain4<D, P, SYS, T, B0, B1, B2, NTH>(I, c.bx * B0, c.by * B1, c.bz * B2, c.bx, c.by, c.bz, tin);
+    else
+        fixed_chain<D, P, SYS, T, B0, B1, B2, NTH>(I, c.bx * B0, c.by * B1, c.bz * B2, c.bx, c.by, c.bz, tin);
 }
 
 // Fixed-shape step kernel on a persistent grid (blocks walk tiles
@@ -890,7 +1085,7 @@ __global__ void __launch_bounds__(NTH, MINB) step_kernel_fixed(const __grid_cons
         // (one buffer: the look-back first, so that its summary loads do not
         // queue behind the tile's copies; the other resident blocks keep
         // HBM busy meanwhile)
-        if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH>(I, t, tin);
+        if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH, false>(I, t, tin);
         if (STG == 1) fixed_load<D, P, SYS, T, B0, B1, B2, NTH>(I, t, cur);
         const int tn = t + gridDim.x;
         if (STG == 2 && tn < ntiles) {
@@ -924,7 +1119,7 @@ __global__ void __launch_bounds__(NTH, MINB)
     for (int i = 0; w < nwork; ++i, w += gridDim.x) {
         const Inst& I = insts[wk.x];
         T* const cur = (i & 1) ? s1 : s0;
-        if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH>(I, wk.y, tin);
+        if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH, true>(I, wk.y, tin);
         if (STG == 1) fixed_load<D, P, SYS, T, B0, B1, B2, NTH>(I, wk.y, cur);
         const int wn = w + gridDim.x;
         int2 wkn = wk;
@@ -955,7 +1150,7 @@ namespace kin {
 template <int D, int P, int SYS, typename T, int B0, int B1, int B2, int NTH>
 __device__ __forceinline__ void fixed_tile_1buf(const Inst& I, int t, T* s, T* tin)
 {
-    if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH>(I, t, tin);
+    if (I.mode == 0) fixed_chain_tile<D, P, SYS, T, B0, B1, B2, NTH, true>(I, t, tin);
     fixed_load<D, P, SYS, T, B0, B1, B2, NTH>(I, t, s);
     cp_wait_all();
     __syncthreads();

@@ -20,12 +20,12 @@ static StepKernel pick(int prec)
     X(1, kEuler, float, 8, 2, 2, 128, 6, 3)         \
     X(1, kEuler, float, 4, 4, 2, 128, 6, 3)         \
     X(1, kEuler, float, 8, 4, 2, 256, 3, 1)         \
-    X(1, kEuler, float, 4, 4, 4, 320, 3, 1)         \
+    X(1, kEuler, float, 4, 4, 4, 256, 3, 1)         \
     X(1, kMaxwell, float, 4, 4, 2, 128, 4, 2)       \
     X(1, kMaxwell, float, 8, 2, 2, 128, 4, 2)       \
     X(1, kMaxwell, float, 4, 2, 2, 64, 8, 4)        \
     X(1, kMaxwell, float, 8, 4, 2, 256, 2, 1)       \
-    X(1, kMaxwell, float, 4, 4, 4, 256, 2, 1)
+    X(1, kMaxwell, float, 4, 4, 4, 288, 2, 1)
 
 FixedKernel fixed_kernel_d3(int degree, int system, int prec, const int B[3], int stages)
 {
