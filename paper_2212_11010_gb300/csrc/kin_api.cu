@@ -73,6 +73,9 @@ struct kin_ctx {
     void* sxtr[2][3] = {};
     std::vector<double> sx_hrec;      // FP64 records [velocity][sx_stride], passed in the sweep parameters
     SxPlan sx_plan = {};
+    void* sxz = nullptr;              // split sweep (2D, FP32): records; NULL when they did not fit the budget
+    int sxz_parity = 0;
+    bool sxz_ready = false;           // the records are those of f
     int sx_stride = 0;
     // tetrahedral meshes
     bool tet = false;
@@ -602,6 +605,13 @@ static kin_status sx_step(kin_ctx* c)
         for (int a = 0; a < 3; ++a) S.tr_out[a] = c->sxtr[0][a];
         KIN_CUDA(c, sx_launch_trace0(S, prec, c->stream));
     }
+    if (c->sxz) {
+        KIN_CUDA(c, sx_split_step(S, c->sx_hrec.data(), c->sx_stride, c->sx_plan, c->sxz, c->sxz_parity, c->sxz_ready,
+                                  c->iters, c->sxtr, c->stream));
+        c->sxz_parity ^= 1;
+        c->sxz_ready = true;
+        return KIN_OK;
+    }
     for (int it = 1; it <= c->iters; ++it) {
         for (int a = 0; a < 3; ++a) {
             S.tr_in[a] = c->sxtr[(it - 1) & 1][a];
@@ -878,6 +888,11 @@ kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, 
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess) {
             e = sx_sweep_plan(sx_args(c), c->precision == KIN_FP32, &c->sx_plan);
+            // (the records are an option: without room for them the one-kernel sweep runs)
+            if (e == cudaSuccess && c->dim == 2 && c->precision == KIN_FP32 &&
+                dev_alloc(c, sx_split_bytes(sx_args(c)), &c->sxz) == KIN_OK)
+                e = sx_split_plan(sx_args(c), &c->sx_plan);
+            c->err.clear();
             c->grid = c->sx_plan.split ? c->sx_plan.bpv : c->nvel * c->sx_plan.bpv;
             c->threads = c->sx_plan.threads;
             c->smem = (int)c->sx_plan.smem;
@@ -1423,6 +1438,7 @@ kin_status kin_set_state(kin_ctx* c, const double* W, size_t n_values, int on_de
         KIN_CUDA(c, tet_launch_init(tet_args(c), src, c->precision == KIN_FP32, c->stream));
     } else if (c->simplex) {
         KIN_CUDA(c, sx_launch_init(sx_args(c), src, c->precision == KIN_FP32, c->stream));
+        c->sxz_ready = false;
     } else {
         KIN_CUDA(c, launch_init(point_args(c), src, c->f, c->precision == KIN_FP32, c->stream));
         st = launch_step(c, 1);
@@ -1448,6 +1464,7 @@ kin_status kin_set_kinetic(kin_ctx* c, const void* f, size_t n_values, int on_de
         return fail(c, KIN_EINVAL, "expected %zu values, got %zu", (size_t)c->npop * c->nodes, n_values);
     KIN_CUDA(c, cudaMemcpyAsync(c->f, f, n_values * c->esize,
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    c->sxz_ready = false;
     if (!c->simplex && !c->tet) {
         st = launch_step(c, 1);
         if (st) return st;
@@ -1474,6 +1491,7 @@ kin_status kin_set_kinetic_async(kin_ctx* c, const void* f, size_t n_values, voi
     // the interface summaries of the new f are computed by the next step
     // (kin_step, kin_batch_step) or diagnostic that needs them
     if (!c->simplex && !c->tet) c->sum_stale = true;
+    c->sxz_ready = false;
     c->have_state = true;
     return KIN_OK;
 }

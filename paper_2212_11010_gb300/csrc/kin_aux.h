@@ -13,10 +13,10 @@ constexpr int kDiagBlocks = 304;   // 2 x 152 SMs
 struct Inst;
 
 // Constants of the relaxation in both precisions, computed once on the host:
-// one FP64 operation of a warp occupies the SM's FP64 units for 16 cycles, so
-// the conversions and the division 1 / (2 lambda) at the head of every tile (or
-// thread) took up to a quarter of a kernel's time: a batch step of 24 uneven 2D
-// problems (FP32) ran 0.88 ms with them.
+// one FP64 operation of a warp occupies the SM's FP64 units for 16 cycles, and
+// the conversions and the division 1 / (2 lambda) stood at the head of every
+// tile of a batch and of every thread of the pointwise relaxations (0.5 to 2%
+// of a step).
 template <typename T>
 struct RelaxK {
     T omega, om1, gm1, inv2l, inv4l, mu, adv[3];     // om1 = 1 - omega, gm1 = gamma - 1, inv2l = 1 / (2 lambda)
@@ -119,12 +119,22 @@ struct SxPlan {
     int threads, bpv, split, occupancy;
     int brick;           // 2 x 2 x 2 cells per lane and wave (3D, p = 1, FP32)
     size_t smem;
+    int split_bpv;       // split sweep (2D, FP32): blocks per velocity of the chain
+    size_t split_smem;
 };
 int sx_sweep_shape(const SxArgs& a, int prec, SxPlan* plan);   // host only: 0 if no shape fits
 cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan);
 cudaError_t sx_launch_sweep(const SxArgs& a, int prec, const double* hrec, int rstride, const SxPlan& plan,
                             cudaStream_t st);
 cudaError_t sx_launch_relax(const SxArgs& a, int prec, cudaStream_t st);
+// Split sweep (2D, FP32): its plan (after sx_sweep_plan), the bytes of its two
+// sets of records Z, and one step; this step's set is number 'parity' (already
+// holding the records of f^n when ready), the other receives the next step's;
+// tr[i][axis] are the trace buffers, with iterate 0 in tr[0] when iters == 1.
+cudaError_t sx_split_plan(const SxArgs& a, SxPlan* plan);
+size_t sx_split_bytes(const SxArgs& a);
+cudaError_t sx_split_step(const SxArgs& a, const double* hrec, int rstride, const SxPlan& plan, void* Z, int parity,
+                          int ready, int iters, void* const (*tr)[3], cudaStream_t st);
 cudaError_t sx_launch_init(const SxArgs& a, const double* W, int prec, cudaStream_t st);
 
 // ---- tetrahedral meshes (kin_tet.cu) ----

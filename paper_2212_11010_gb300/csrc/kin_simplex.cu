@@ -26,6 +26,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace kin {
@@ -1043,63 +1044,434 @@ __global__ void __launch_bounds__(32) sx_brick_kernel(const __grid_constant__ Sx
     else sx_brick_velocity<3>(A, lb, sm);
 }
 
-// Relaxation with the d + 1 velocity equilibria: M_{k,v} = sum_j Minv[k][j] rhs_j,
-// rhs = (W_v, Q^1_v, ..., Q^d_v) (eq. maxwell_def).
+// ---------------------------------------------------------------------------
+// split sweep: 2D, FP32
+// ---------------------------------------------------------------------------
+
+// A 2D mesh has few problems (768 for 64 subdomains of the vortex), so a sweep
+// is as long as its chain: 63 waves of one warp, 1,800 cycles each with the
+// whole cell solve in the chain (57 us per iterate at p = 2).  But of
+//   f* = t + A^{-1} (W_cell (f^n - t) + sum_a nu_a E_a W_perp (tr_a - t))
+// the next cell needs only the outflow nodes, and the f^n part of those is known
+// before the sweep starts.  So a step is
+//   local   for every cell, t and t + A^{-1} W_cell (f^n - t) at the outflow
+//           nodes (one record Z per population and cell), all cells at once --
+//           only after f was set: otherwise the step before has left them;
+//   chain   K sweeps over the records: per cell 2 (p + 1) inflow values, a
+//           (2p + 1) x 2(p + 1) matrix and 2p + 1 outflow values (p = 2: 30
+//           FMAs instead of 87); the last one leaves the outflow values in Z;
+//   finish  for every cell, the full solve with its final inflow, f^{n+1} =
+//           2 f* - f^n, the relaxation and the next step's record, all cells
+//           at once: f is read and written once.
+// Both parts vanish for a constant state, so it is kept exactly, as in the
+// one-kernel form.
+//   Measured (20 steps with set-up and read-back, before -> now): 256^2 cells,
+// p = 2 3.77 -> 2.18 ms; 378^2, 9-cell subdomains, p = 3 15.0 -> 5.6; 320 x 80,
+// 40-cell subdomains, p = 3 6.7 -> 2.2; 384^2, 8-cell subdomains, p = 1 5.5 ->
+// 2.5; 64^2, p = 1 1.87 -> 1.18.  What bounds it: the waves' latency (63 of them,
+// three times a step) and the finish, 40 us cold, by its shared-memory traffic.
+template <int P>
+struct SxSplit {
+    static constexpr int NP = P + 1, NN = NP * NP, TN = NP, NO = 2 * TN - 1, NI = 2 * TN;
+    static constexpr int ZS = (NO + 1 + 3) / 4 * 4;      // floats per record: t, outflow nodes
+    SxArgs S;
+    float *Z, *Znext;                                    // records of this step, and of the next one
+    int bpv;
+    SxDiv div_nsub, div_ns0, div_n0, div_L0, div_L1;
+    float gm[3][NO][NI];                                 // outflow node <- inflow value (axis DEP, then the other)
+    float aw[3][NO][NN];                                 // outflow node <- f^n - t
+    float ainv[3][NN * NN], wcell[NN], face[3][2][TN];
+};
+
+// Axis along which velocity k's chain runs, and the record's slot of each
+// outflow node: the nodes of the face along that axis, then the rest of the other
+// face (they share a corner).
+__host__ __device__ constexpr int sp_dep(int k) { return k == 0 ? 0 : 1; }
+__host__ __device__ constexpr int sp_out(int k, int a, int P) { return sx_sign(2, k, a) > 0 ? P : 0; }
+template <int P>
+__host__ __device__ constexpr int sp_slot(int k, int a, int tt)
+{
+    const int dep = sp_dep(k), od = sp_out(k, dep, P);
+    if (a == dep) return tt;
+    return tt == od ? sp_out(k, 1 - dep, P) : P + 1 + (tt < od ? tt : tt - 1);
+}
+template <int P>
+__host__ __device__ constexpr int sp_node(int k, int slot)
+{
+    constexpr int NP = P + 1;
+    const int dep = sp_dep(k), od = sp_out(k, dep, P), ot = sp_out(k, 1 - dep, P);
+    if (slot < NP) return sx_node<2, NP>(dep, od, slot);
+    const int r = slot - NP, tt = r < od ? r : r + 1;
+    return sx_node<2, NP>(1 - dep, ot, tt);
+}
+
+template <int P>
+__global__ void __launch_bounds__(64 * (P + 1)) sx_local_kernel(const __grid_constant__ SxSplit<P> A)
+{
+    using SP = SxSplit<P>;
+    constexpr int NN = SP::NN, NO = SP::NO, ZS = SP::ZS, NNP = NN | 1, ZP = ZS + 1, NT = 32 * (NO + 1);
+    __shared__ float u[32 * NNP], zr[32 * ZP];
+    const int s = threadIdx.x >> 5, c = threadIdx.x & 31;          // warp: a slot; lanes: cells
+    const long long cells = A.S.nodes / NN;
+    const int pop = blockIdx.y, k = pop / A.S.m;
+    const float* f = static_cast<const float*>(A.S.f) + (long long)pop * A.S.nodes;
+    for (long long c0 = blockIdx.x * 32LL; c0 < cells; c0 += gridDim.x * 32LL) {
+        const int nc = (int)(cells - c0 < 32 ? cells - c0 : 32);
+        for (int e = threadIdx.x; e < nc * NN; e += NT) u[(e / NN) * NNP + e % NN] = f[c0 * NN + e];
+        __syncthreads();
+        const float t = u[c * NNP];
+        float z = t;
+        if (s > 0) {
+            float acc = 0.0f;
+#pragma unroll
+            for (int j = 1; j < NN; ++j) acc = fmaf(A.aw[k][s - 1][j], u[c * NNP + j] - t, acc);
+            z = acc + t;
+        }
+        zr[c * ZP + s] = z;
+        __syncthreads();
+        float* Z = A.Z + ((long long)pop * cells + c0) * ZS;
+        for (int e = threadIdx.x; e < nc * ZS; e += NT) Z[e] = zr[(e / ZS) * ZP + e % ZS];
+        __syncthreads();
+    }
+}
+
+// Problems that a block of nt lanes takes side by side on lanes of n0 columns
+// each: as many as fit, while their transverse faces (2 Ld TN values each)
+// stay within 32 KB.
+__host__ __device__ inline int chain_groups(int nt, int n0, int Ld, int TN)
+{
+    const int fit = nt / n0, room = 4096 / (Ld * TN);
+    return fit < 1 ? 1 : (fit <= room ? fit : (room < 1 ? 1 : room));
+}
+
+// One velocity's chain: the lanes and the skew of sx_sweep_velocity (D = 2) on
+// records, problem after problem.  What a wave needs besides its record is
+// moved out of the waves -- a problem's inflow along both axes is loaded before
+// its first, its outflow traces are stored after its last -- because in a wave
+// it is one lane's work that the whole warp waits for (with it in the waves they
+// took 1,000 to 1,400 cycles).
+template <int P, int KV>
+__device__ __forceinline__ void sx_chain_velocity(const SxSplit<P>& A, const int lb, float* sm)
+{
+    using SP = SxSplit<P>;
+    constexpr int NP = SP::NP, NN = SP::NN, TN = SP::TN, ZS = SP::ZS;
+    constexpr int NEP = sx_pad_odd(ZS, 4), TNP = sx_pad_odd(TN, TN == 4 ? 4 : 1);
+    constexpr int DEP = sp_dep(KV), TA = 1 - DEP, SGD = sx_sign(2, KV, DEP), SGT = sx_sign(2, KV, TA);
+    constexpr bool X0 = SGT != 0;
+    constexpr int NO = X0 ? SP::NO : TN, NI = X0 ? SP::NI : TN;
+    const SxArgs& S = A.S;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int n0 = S.L[TA], Ld = S.L[DEP];
+    const int G = chain_groups(nt, n0, Ld, TN), grp = tid / n0, ln = tid - grp * n0;
+    const int lt = SGT < 0 ? n0 - 1 - ln : ln;
+    const int skew = X0 ? ln : 0, waves = Ld + (X0 ? n0 - 1 : 0);
+    const int nsub = S.NS[0] * S.NS[1], nprob = S.m * nsub;
+    const long long cells = S.nodes / NN;
+    const float* f = static_cast<const float*>(S.f);
+    float* const ring = sm;                                // [2][lane][NEP]
+    float* const xs = ring + 2 * nt * NEP;                 // exchange [2][lane][TNP]
+    float* const tin = xs + 2 * nt * TNP + grp * (2 * Ld * TN), *const tout = tin + Ld * TN;
+    auto sync = [&]() {
+        if (nt > 32) __syncthreads();
+        else __syncwarp();
+    };
+    auto xslot = [&](int par) { return xs + (par * nt + tid) * TNP; };
+
+    for (int base = lb * G; base < nprob; base += A.bpv * G) {
+        const int pid = base + grp;
+        const bool has = grp < G && pid < nprob;
+        const int v = sx_div(has ? pid : 0, A.div_nsub), sub = (has ? pid : 0) - v * nsub;
+        int s[2];
+        s[1] = sx_div(sub, A.div_ns0);
+        s[0] = sub - s[1] * S.NS[0];
+        const int pop = KV * S.m + v, gt = s[TA] * n0 + lt;
+        auto along = [&](int od) { return s[DEP] * Ld + (SGD < 0 ? Ld - 1 - od : od); };
+        // value tt of the inflow across axis a's interface at transverse cell gc
+        auto inflow = [&](int a, int gc, int tt) {
+            const int sg = a == DEP ? SGD : SGT;
+            if (S.from_f) {
+                // iterate 0 of eq. ibvp: f^n on the outflow face of the upwind cell
+                int g = s[a] * S.L[a] + (sg > 0 ? -1 : S.L[a]);
+                if (g < 0) g += S.n[a];
+                if (g >= S.n[a]) g -= S.n[a];
+                const int cell = a == 0 ? gc * S.n[0] + g : g * S.n[0] + gc;
+                return f[(long long)pop * S.nodes + (long long)cell * NN + sx_node<2, NP>(a, sg > 0 ? P : 0, tt)];
+            }
+            int sup = s[a] - sg;
+            if (sup < 0) sup += S.NS[a];
+            if (sup >= S.NS[a]) sup -= S.NS[a];
+            return static_cast<const float*>(S.tr_in[a])[((long long)pop * S.NS[a] + sup) * S.glines[a] +
+                                                          (long long)gc * TN + tt];
+        };
+        float pd[TN];                                      // outflow face along DEP of the wave before
+#pragma unroll
+        for (int tt = 0; tt < TN; ++tt) pd[tt] = has ? inflow(DEP, gt, tt) : 0.0f;
+        if (X0 && has)
+            for (int e = ln; e < Ld * TN; e += n0) tin[e] = inflow(TA, along(e / TN), e % TN);
+        const int c0 = DEP == 0 ? gt * S.n[0] + along(0) : along(0) * S.n[0] + gt;
+        float* const z0 = A.Z + ((long long)pop * cells + c0) * ZS;
+        const long long zstep = (long long)SGD * (DEP == 0 ? 1 : S.n[0]) * ZS;
+        auto fetch = [&](int W) {
+            const int q = W - skew;
+            if (has && q >= 0 && q < Ld) {
+                float* d = ring + ((W & 1) * nt + tid) * NEP;
+                const float* src = z0 + q * zstep;
+#pragma unroll
+                for (int e = 0; e < ZS; e += 4) cp16_g2s(d + e, src + e);
+            }
+            cp_commit();
+        };
+        fetch(0);
+        sync();                                            // tin is there for the group's first lane
+        for (int W = 0; W < waves; ++W) {
+            fetch(W + 1);
+            cp_wait_group<1>();
+            const int q = W - skew;
+            if (has && q >= 0 && q < Ld) {
+                float z[ZS], g[NI], o[NO];
+                sx_lds<ZS, true>(ring + ((W & 1) * nt + tid) * NEP, z);
+#pragma unroll
+                for (int tt = 0; tt < TN; ++tt) g[tt] = pd[tt] - z[0];
+                if constexpr (X0) {
+                    const float* src = ln == 0 ? tin + q * TN : xslot((W & 1) ^ 1) - TNP;
+#pragma unroll
+                    for (int tt = 0; tt < TN; ++tt) g[TN + tt] = src[tt] - z[0];
+                }
+#pragma unroll
+                for (int sl = 0; sl < NO; ++sl) o[sl] = fmaf(A.gm[KV][sl][0], g[0], z[1 + sl]);
+#pragma unroll
+                for (int j = 1; j < NI; ++j)
+#pragma unroll
+                    for (int sl = 0; sl < NO; ++sl) o[sl] = fmaf(A.gm[KV][sl][j], g[j], o[sl]);
+#pragma unroll
+                for (int tt = 0; tt < TN; ++tt) pd[tt] = o[tt];
+                if constexpr (X0) {
+                    float* d = ln == n0 - 1 ? tout + q * TN : xslot(W & 1);
+#pragma unroll
+                    for (int tt = 0; tt < TN; ++tt) d[tt] = o[sp_slot<P>(KV, TA, tt)];
+                }
+                if (S.final_iter) {
+#pragma unroll
+                    for (int sl = 0; sl < NO; ++sl) z[1 + sl] = o[sl];
+                    sx_st<ZS>(z0 + q * zstep, z);
+                }
+            }
+            sync();
+        }
+        if (!S.final_iter && has) {
+            float* tr = static_cast<float*>(S.tr_out[DEP]) + ((long long)pop * S.NS[DEP] + s[DEP]) * S.glines[DEP] +
+                        (long long)gt * TN;
+#pragma unroll
+            for (int tt = 0; tt < TN; ++tt) tr[tt] = pd[tt];
+            if constexpr (X0) {
+                float* tx = static_cast<float*>(S.tr_out[TA]) + ((long long)pop * S.NS[TA] + s[TA]) * S.glines[TA];
+                for (int e = ln; e < Ld * TN; e += n0) tx[(long long)along(e / TN) * TN + e % TN] = tout[e];
+            }
+        }
+        sync();                                            // tin and tout may be filled again
+    }
+    cp_wait_group<0>();
+}
+
+template <int P, int MAXT>
+__global__ void __launch_bounds__(MAXT) sx_chain_kernel(const __grid_constant__ SxSplit<P> A)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float* sm = reinterpret_cast<float*>(smem_raw);
+    const int k = (int)blockIdx.x / A.bpv, lb = (int)blockIdx.x % A.bpv;
+    if (k == 0) sx_chain_velocity<P, 0>(A, lb, sm);
+    else if (k == 1) sx_chain_velocity<P, 1>(A, lb, sm);
+    else sx_chain_velocity<P, 2>(A, lb, sm);
+}
+
+// (the velocities with a transverse inflow run along y on lanes along x)
+template <int P>
+static size_t chain_smem(int nt, const int* L)
+{
+    constexpr int TN = P + 1, NEP = sx_pad_odd(SxSplit<P>::ZS, 4), TNP = sx_pad_odd(TN, TN == 4 ? 4 : 1);
+    return sizeof(float) * ((size_t)2 * nt * (NEP + TNP) + (size_t)chain_groups(nt, L[0], L[1], TN) * 2 * L[1] * TN);
+}
+
+// Relaxation of one node's populations with the d + 1 velocity equilibria:
+// M_{k,v} = sum_j Minv[k][j] rhs_j, rhs = (W_v, Q^1_v, ..., Q^d_v) (eq. maxwell_def).
 template <int D, int SYS, typename T>
-__global__ void sx_relax_kernel(const __grid_constant__ SxArgs S)
+__device__ __forceinline__ void sx_relax_node(const SxArgs& S, T* fk)
 {
     constexpr int M = nvars(D, SYS);
     constexpr int NV = D + 1;
-    T* f = static_cast<T*>(S.f);
     const RelaxK<T>& RK = relax_k<T>(S.rx);
     auto minv = [&](int i, int j) -> T {
         if constexpr (sizeof(T) == 4) return S.minvf[i * NV + j];
         else return S.minv[i * NV + j];
     };
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.nodes;
-         i += (long long)gridDim.x * blockDim.x) {
-        T fk[NV * M];
+    T W[M];
 #pragma unroll
-        for (int p = 0; p < NV * M; ++p) fk[p] = f[(long long)p * S.nodes + i];
-        T W[M];
+    for (int v = 0; v < M; ++v) {
+        Acc<T> acc;
+#pragma unroll
+        for (int kk = 0; kk < NV; ++kk) acc.add(fk[kk * M + v]);
+        W[v] = acc.s;
+    }
+    T Q[D][M];
+    if (SYS == kAdvection) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) Q[a][0] = RK.adv[a] * W[0];
+    } else {
+        const T inv = T(1) / W[0];
+        T ke = 0;
+#pragma unroll
+        for (int b = 0; b < D; ++b) ke = fma(W[1 + b], W[1 + b], ke);
+        const T pr = RK.gm1 * (W[1 + D] - T(0.5) * ke * inv);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const T ua = W[1 + a] * inv;
+            Q[a][0] = W[1 + a];
+#pragma unroll
+            for (int b = 0; b < D; ++b) Q[a][1 + b] = W[1 + b] * ua + (b == a ? pr : T(0));
+            Q[a][1 + D] = (W[1 + D] + pr) * ua;
+        }
+    }
+#pragma unroll
+    for (int kk = 0; kk < NV; ++kk)
 #pragma unroll
         for (int v = 0; v < M; ++v) {
-            Acc<T> acc;
+            T mk = minv(kk, 0) * W[v];
 #pragma unroll
-            for (int kk = 0; kk < NV; ++kk) acc.add(fk[kk * M + v]);
-            W[v] = acc.s;
+            for (int a = 0; a < D; ++a) mk = fma(minv(kk, 1 + a), Q[a][v], mk);
+            T& fv = fk[kk * M + v];
+            fv = S.rx.two ? fma(T(2), mk, -fv) : RK.omega * mk + RK.om1 * fv;
         }
-        T Q[D][M];
-        if (SYS == kAdvection) {
+}
+
+// Threads: node-major over 32 cells, so that a warp's node, and with it every
+// coefficient, is uniform.
+template <int P, int SYS>
+__global__ void __launch_bounds__(32 * (P + 1) * (P + 1)) sx_finish_kernel(const __grid_constant__ SxSplit<P> A)
+{
+    using SP = SxSplit<P>;
+    constexpr int NP = SP::NP, NN = SP::NN, TN = SP::TN, ZS = SP::ZS, NNP = NN | 1, NT = 32 * NN;
+    constexpr int M = nvars(2, SYS), NPOP = 3 * M;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float* const u = reinterpret_cast<float*>(smem_raw);         // [pop][cell][NNP]
+    float* const r = u + NPOP * 32 * NNP;                         // [pop][node][cell]
+    float* const tr = r + NPOP * NN * 32;                         // [pop][axis][face node][cell]
+    const SxArgs& S = A.S;
+    const int n = threadIdx.x >> 5, c = threadIdx.x & 31;
+    const long long cells = S.nodes / NN;
+    float* const f = static_cast<float*>(S.f);
+    for (long long c0 = blockIdx.x * 32LL; c0 < cells; c0 += gridDim.x * 32LL) {
+        const int nc = (int)(cells - c0 < 32 ? cells - c0 : 32);
+        // (every load by cp.async: a dozen loops of loads waited for one by one
+        // took most of the kernel's time, 44 us for 256^2 cells at p = 2)
+        if ((int)threadIdx.x < nc * NN) {
 #pragma unroll
-            for (int a = 0; a < D; ++a) Q[a][0] = RK.adv[a] * W[0];
-        } else {
-            const T inv = T(1) / W[0];
-            T ke = 0;
+            for (int pop = 0; pop < NPOP; ++pop)
+                cp_small_g2s<4>(u + (pop * 32 + threadIdx.x / NN) * NNP + threadIdx.x % NN,
+                                f + (long long)pop * S.nodes + c0 * NN + threadIdx.x);
+        }
+        for (int e = threadIdx.x; e < NPOP * 2 * 32; e += NT) {
+            const int cc = e & 31, a = (e >> 5) & 1, pop = e >> 6, k = pop / M, sg = sx_sign(2, k, a);
+            if (sg == 0 || cc >= nc) continue;
+            const int cell = (int)c0 + cc, gy = sx_div(cell, A.div_n0), gx = cell - gy * S.n[0];
+            const int ga = a == 0 ? gx : gy, sub = sx_div(ga, a == 0 ? A.div_L0 : A.div_L1), la = ga - sub * S.L[a];
+            float* const d = tr + (pop * 2 + a) * TN * 32 + cc;
+            if (la == (sg > 0 ? 0 : S.L[a] - 1)) {
+                int sup = sub - sg;
+                if (sup < 0) sup += S.NS[a];
+                if (sup >= S.NS[a]) sup -= S.NS[a];
+                const float* p = static_cast<const float*>(S.tr_in[a]) + ((long long)pop * S.NS[a] + sup) * S.glines[a] +
+                                 (long long)(a == 0 ? gy : gx) * TN;
 #pragma unroll
-            for (int b = 0; b < D; ++b) ke = fma(W[1 + b], W[1 + b], ke);
-            const T pr = RK.gm1 * (W[1 + D] - T(0.5) * ke * inv);
+                for (int tt = 0; tt < TN; ++tt) cp_small_g2s<4>(d + tt * 32, p + tt);
+            } else {
+                const float* p = A.Z + ((long long)pop * cells + cell - (a == 0 ? sg : sg * S.n[0])) * ZS + 1;
 #pragma unroll
-            for (int a = 0; a < D; ++a) {
-                const T ua = W[1 + a] * inv;
-                Q[a][0] = W[1 + a];
-#pragma unroll
-                for (int b = 0; b < D; ++b) Q[a][1 + b] = W[1 + b] * ua + (b == a ? pr : T(0));
-                Q[a][1 + D] = (W[1 + D] + pr) * ua;
+                for (int tt = 0; tt < TN; ++tt) cp_small_g2s<4>(d + tt * 32, p + sp_slot<P>(k, a, tt));
             }
         }
+        cp_commit();
+        cp_wait_all();
+        __syncthreads();
+        const int jx = n % NP, jy = n / NP;
 #pragma unroll
-        for (int kk = 0; kk < NV; ++kk)
+        for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int v = 0; v < M; ++v) {
-                T mk = minv(kk, 0) * W[v];
+                const int pop = k * M + v;
+                const float t = u[(pop * 32 + c) * NNP];
+                float x = n == 0 ? 0.0f : A.wcell[n] * (u[(pop * 32 + c) * NNP + n] - t);
 #pragma unroll
-                for (int a = 0; a < D; ++a) mk = fma(minv(kk, 1 + a), Q[a][v], mk);
-                T& fv = fk[kk * M + v];
-                fv = S.rx.two ? fma(T(2), mk, -fv) : RK.omega * mk + RK.om1 * fv;
+                for (int a = 0; a < 2; ++a) {
+                    const int sg = sx_sign(2, k, a);
+                    if (sg == 0 || (a == 0 ? jx : jy) != (sg > 0 ? 0 : P)) continue;
+                    const int tt = a == 0 ? jy : jx;
+                    x = fmaf(A.face[k][a][tt], tr[((pop * 2 + a) * TN + tt) * 32 + c] - t, x);
+                }
+                r[(pop * NN + n) * 32 + c] = x;
             }
+        __syncthreads();
+        float fk[NPOP];
 #pragma unroll
-        for (int p = 0; p < NV * M; ++p) f[(long long)p * S.nodes + i] = fk[p];
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+                const int pop = k * M + v;
+                float x = A.ainv[k][n * NN] * r[pop * NN * 32 + c];
+#pragma unroll
+                for (int j = 1; j < NN; ++j) x = fmaf(A.ainv[k][n * NN + j], r[(pop * NN + j) * 32 + c], x);
+                x += u[(pop * 32 + c) * NNP];
+                fk[pop] = fmaf(2.0f, x, -u[(pop * 32 + c) * NNP + n]);
+            }
+        sx_relax_node<2, SYS, float>(S, fk);
+        __syncthreads();
+#pragma unroll
+        for (int pop = 0; pop < NPOP; ++pop) u[(pop * 32 + c) * NNP + n] = fk[pop];
+        __syncthreads();
+        if ((int)threadIdx.x < nc * NN) {
+#pragma unroll
+            for (int pop = 0; pop < NPOP; ++pop)
+                f[(long long)pop * S.nodes + c0 * NN + threadIdx.x] =
+                    u[(pop * 32 + threadIdx.x / NN) * NNP + threadIdx.x % NN];
+        }
+        // the next step's records while f^{n+1} is here (sx_local_kernel)
+        float* const zr = r;                                      // [pop][cell][ZS + 1]
+        constexpr int NO = SP::NO, ZP = ZS + 1;
+        static_assert(ZP <= NN + 2 * TN, "the records fit where the right-hand sides and faces were");
+        if (n <= NO) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int v = 0; v < M; ++v) {
+                    const int pop = k * M + v;
+                    const float* const uc = u + (pop * 32 + c) * NNP;
+                    float acc = 0.0f;
+                    if (n > 0)
+#pragma unroll
+                        for (int j = 1; j < NN; ++j) acc = fmaf(A.aw[k][n - 1][j], uc[j] - uc[0], acc);
+                    zr[(pop * 32 + c) * ZP + n] = n > 0 ? acc + uc[0] : uc[0];
+                }
+        }
+        __syncthreads();
+        for (int pop = 0; pop < NPOP; ++pop)
+            for (int e = threadIdx.x; e < nc * ZS; e += NT)
+                A.Znext[((long long)pop * cells + c0) * ZS + e] = zr[(pop * 32 + e / ZS) * ZP + e % ZS];
+        __syncthreads();
+    }
+}
+
+template <int D, int SYS, typename T>
+__global__ void sx_relax_kernel(const __grid_constant__ SxArgs S)
+{
+    constexpr int NPOP = (D + 1) * nvars(D, SYS);
+    T* f = static_cast<T*>(S.f);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S.nodes;
+         i += (long long)gridDim.x * blockDim.x) {
+        T fk[NPOP];
+#pragma unroll
+        for (int p = 0; p < NPOP; ++p) fk[p] = f[(long long)p * S.nodes + i];
+        sx_relax_node<D, SYS>(S, fk);
+#pragma unroll
+        for (int p = 0; p < NPOP; ++p) f[(long long)p * S.nodes + i] = fk[p];
     }
 }
 
@@ -1313,6 +1685,119 @@ static cudaError_t wave_launch(const SxArgs& a, const double* hrec, int rstride,
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// ---- split sweep (2D, FP32): one step from f^n to f^{n+1} ----
+template <int P>
+static cudaError_t split_step(SxArgs a, const double* hrec, int rstride, const SxPlan& plan, float* Z, float* Znext,
+                              bool ready, int iters, void* const (*tr)[3], cudaStream_t st)
+{
+    using SP = SxSplit<P>;
+    constexpr int NN = SP::NN, TN = SP::TN, NO = SP::NO, NP = SP::NP;
+    static_assert(sizeof(SP) <= 32000, "parameters exceed the kernel parameter limit");
+    SP w;
+    memset(&w, 0, sizeof w);
+    w.Z = Z;
+    w.Znext = Znext;
+    w.bpv = plan.split_bpv;
+    w.div_nsub = sx_div_make(a.NS[0] * a.NS[1]);
+    w.div_ns0 = sx_div_make(a.NS[0]);
+    w.div_n0 = sx_div_make(a.n[0]);
+    w.div_L0 = sx_div_make(a.L[0]);
+    w.div_L1 = sx_div_make(a.L[1]);
+    for (int j = 0; j < NN; ++j) w.wcell[j] = (float)hrec[NN * NN + j];
+    for (int k = 0; k < 3; ++k) {
+        const double* rec = hrec + (size_t)k * rstride;
+        const double* fc = rec + NN * NN + NN;
+        for (int e = 0; e < NN * NN; ++e) w.ainv[k][e] = (float)rec[e];
+        for (int ax = 0; ax < 2; ++ax)
+            for (int t = 0; t < TN; ++t) w.face[k][ax][t] = (float)fc[ax * TN + t];
+        const bool both = sx_sign(2, k, 1 - sp_dep(k)) != 0;
+        for (int s = 0; s < (both ? NO : TN); ++s) {
+            const int n = sp_node<P>(k, s);
+            for (int j = 0; j < NN; ++j) w.aw[k][s][j] = (float)(rec[n * NN + j] * rec[NN * NN + j]);
+            for (int q = 0; q < (both ? 2 : 1); ++q) {
+                const int ax = q == 0 ? sp_dep(k) : 1 - sp_dep(k);
+                for (int t = 0; t < TN; ++t)
+                    w.gm[k][s][q * TN + t] =
+                        (float)(rec[n * NN + sx_node<2, NP>(ax, sx_sign(2, k, ax) > 0 ? 0 : P, t)] * fc[ax * TN + t]);
+            }
+        }
+    }
+    w.S = a;
+    const long long groups = (a.nodes / NN + 31) / 32;
+    const unsigned gx = (unsigned)(groups < 1024 ? groups : 1024);
+    cudaError_t e = cudaSuccess;
+    if (!ready) {
+        sx_local_kernel<P><<<dim3(gx, a.npop), 64 * (P + 1), 0, st>>>(w);
+        e = cudaGetLastError();
+    }
+    const void* chain = plan.threads <= 64 ? (const void*)sx_chain_kernel<P, 64> : (const void*)sx_chain_kernel<P, 1024>;
+    void* p[] = {&w};
+    for (int it = 1; it <= iters && e == cudaSuccess; ++it) {
+        for (int ax = 0; ax < 3; ++ax) {
+            w.S.tr_in[ax] = tr[(it - 1) & 1][ax];
+            w.S.tr_out[ax] = tr[it & 1][ax];
+        }
+        w.S.from_f = it == 1 && iters > 1;
+        w.S.final_iter = it == iters;
+        e = cudaLaunchKernel(chain, dim3(3 * w.bpv), dim3(plan.threads), p, plan.split_smem, st);
+    }
+    const size_t fsm = sizeof(float) * (size_t)a.npop * 32 * ((NN | 1) + NN + 2 * TN);
+    const unsigned fg = (unsigned)(groups < 152 * 16 ? groups : 152 * 16);
+    const void* fin = a.system == kEuler ? (const void*)sx_finish_kernel<P, kEuler>
+                                         : (const void*)sx_finish_kernel<P, kAdvection>;
+    if (e == cudaSuccess) e = cudaLaunchKernel(fin, dim3(fg), dim3(32 * NN), p, fsm, st);
+    return e;
+}
+
+template <int P>
+static cudaError_t split_plan(const SxArgs& a, SxPlan* plan)
+{
+    constexpr int NN = SxSplit<P>::NN, TN = SxSplit<P>::TN;
+    const void* chain = plan->threads <= 64 ? (const void*)sx_chain_kernel<P, 64> : (const void*)sx_chain_kernel<P, 1024>;
+    plan->split_smem = chain_smem<P>(plan->threads, a.L);
+    int occ = 0, dev = 0, nsm = 0;
+    cudaError_t e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    for (const void* fin : {(const void*)sx_finish_kernel<P, kEuler>, (const void*)sx_finish_kernel<P, kAdvection>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(sizeof(float) * 12 * 32 * ((NN | 1) + NN + 2 * TN)));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, chain, plan->threads, plan->split_smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int G = std::min(chain_groups(plan->threads, a.L[0], a.L[1], TN),
+                           chain_groups(plan->threads, a.L[1], a.L[0], TN));
+    const int nprob = (a.m * a.NS[0] * a.NS[1] + G - 1) / G;
+    int b = occ * nsm / 3;
+    b = b < 1 ? 1 : (b > nprob ? nprob : b);
+    const int per = (nprob + b - 1) / b;
+    plan->split_bpv = (nprob + per - 1) / per;
+    return cudaSuccess;
+}
+
+cudaError_t sx_split_plan(const SxArgs& a, SxPlan* plan)
+{
+    return a.degree == 1 ? split_plan<1>(a, plan) : (a.degree == 2 ? split_plan<2>(a, plan) : split_plan<3>(a, plan));
+}
+
+size_t sx_split_bytes(const SxArgs& a)
+{
+    const int zs = a.degree == 1 ? SxSplit<1>::ZS : (a.degree == 2 ? SxSplit<2>::ZS : SxSplit<3>::ZS);
+    return 2 * sizeof(float) * (size_t)a.npop * (size_t)(a.nodes / a.nn) * zs;
+}
+
+cudaError_t sx_split_step(const SxArgs& a, const double* hrec, int rstride, const SxPlan& plan, void* Z, int parity,
+                          int ready, int iters, void* const (*tr)[3], cudaStream_t st)
+{
+    const size_t half = sx_split_bytes(a) / 2 / sizeof(float);
+    float* z = static_cast<float*>(Z) + (parity ? half : 0);
+    float* zn = static_cast<float*>(Z) + (parity ? 0 : half);
+    if (a.degree == 1) return split_step<1>(a, hrec, rstride, plan, z, zn, ready, iters, tr, st);
+    if (a.degree == 2) return split_step<2>(a, hrec, rstride, plan, z, zn, ready, iters, tr, st);
+    return split_step<3>(a, hrec, rstride, plan, z, zn, ready, iters, tr, st);
 }
 
 template <typename T>
