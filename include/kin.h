@@ -201,9 +201,9 @@ typedef struct {
  * (-,-,+)).  The context then takes kin_set_state, kin_set_kinetic,
  * kin_step, kin_get_state, kin_get_kinetic, kin_diag (mass only),
  * kin_query, kin_sync and kin_destroy; kin_set_boundary and batches return
- * KIN_EINVAL.  Each step is K sweep launches (one thread block per
- * (subdomain, velocity) walking the levels) and one launch for the
- * Crank-Nicolson extrapolation and the relaxation.  Errors: KIN_EINVAL (bad
+ * KIN_EINVAL.  Each step is K sweep launches (thread blocks
+ * walking the levels of their (subdomain, velocity), with the variables
+ * together or apart) and one launch for the relaxation.  Errors: KIN_EINVAL (bad
  * arguments or topology: a neighbour out of range, a face whose vertices are
  * not in the neighbour, a degenerate cell, a cycle in a subdomain's oriented
  * graph), KIN_EBUDGET, KIN_ENOMEM, KIN_ECUDA. */

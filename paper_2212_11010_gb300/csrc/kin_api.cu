@@ -76,6 +76,7 @@ struct kin_ctx {
     void* sxz = nullptr;              // split sweep (2D, FP32): records; NULL when they did not fit the budget
     int sxz_parity = 0;
     bool sxz_ready = false;           // the records are those of f
+    bool sxz_captured = false;        // a step was captured into a graph, which may be replayed at any time
     int sx_stride = 0;
     // tetrahedral meshes
     bool tet = false;
@@ -238,7 +239,7 @@ static void choose_block(const kin_ctx* c, int B[3])
         }
     }
     shrink_block(c, B);
-    if (c->dim < 2) return;
+    if (c->dim < 2 || c->want_stages == 2) return;      // two tile buffers: the small tiles
     int least = B[0];
     for (int a = 1; a < c->dim; ++a) least = std::min(least, B[a]);
     std::vector<int> div[3];
@@ -606,6 +607,14 @@ static kin_status sx_step(kin_ctx* c)
         KIN_CUDA(c, sx_launch_trace0(S, prec, c->stream));
     }
     if (c->sxz) {
+        // a replayed graph advances f without this context knowing: from the
+        // first captured step on, every step computes its own records
+        if (c->stream && !c->sxz_captured) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            KIN_CUDA(c, cudaStreamIsCapturing(c->stream, &cs));
+            c->sxz_captured = cs != cudaStreamCaptureStatusNone;
+        }
+        if (c->sxz_captured) c->sxz_ready = false;
         KIN_CUDA(c, sx_split_step(S, c->sx_hrec.data(), c->sx_stride, c->sx_plan, c->sxz, c->sxz_parity, c->sxz_ready,
                                   c->iters, c->sxtr, c->stream));
         c->sxz_parity ^= 1;

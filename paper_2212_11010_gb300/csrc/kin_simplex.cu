@@ -18,6 +18,9 @@
 //   relaxation   W = sum_k f_k and f_k <- omega M_k(W) + (1 - omega) f_k with
 //                M from the moment system eq. maxwell_def (its inverse is
 //                precomputed in FP64).
+// Two forms take the sweep's place in FP32: bricks of 2 x 2 x 2 cells per lane
+// (3D, degree 1, large meshes; sx_brick_velocity), and in 2D a chain over the
+// outflow nodes alone between two passes over all cells at once (SxSplit).
 #include "kin_aux.h"
 #include "kin_device.cuh"
 #include "kin_init.cuh"
@@ -1757,12 +1760,16 @@ static cudaError_t split_plan(const SxArgs& a, SxPlan* plan)
     constexpr int NN = SxSplit<P>::NN, TN = SxSplit<P>::TN;
     const void* chain = plan->threads <= 64 ? (const void*)sx_chain_kernel<P, 64> : (const void*)sx_chain_kernel<P, 1024>;
     plan->split_smem = chain_smem<P>(plan->threads, a.L);
+    // (set once to a constant where the default 48 KB would not do: contexts
+    // of different sizes share the functions)
     int occ = 0, dev = 0, nsm = 0;
-    cudaError_t e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    for (const void* fin : {(const void*)sx_finish_kernel<P, kEuler>, (const void*)sx_finish_kernel<P, kAdvection>})
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(sizeof(float) * 12 * 32 * ((NN | 1) + NN + 2 * TN)));
+    cudaError_t e = cudaSuccess;
+    if (plan->split_smem > 48 * 1024)
+        e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    constexpr size_t most = sizeof(float) * 12 * 32 * ((NN | 1) + NN + 2 * TN);       // Euler's 12 populations
+    if (e == cudaSuccess && most > 48 * 1024 && a.system == kEuler)
+        e = cudaFuncSetAttribute((const void*)sx_finish_kernel<P, kEuler>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)most);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, chain, plan->threads, plan->split_smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);

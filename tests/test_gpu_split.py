@@ -104,3 +104,29 @@ def test_records_follow_the_state(kin):
         kin.kin_set_kinetic_async(ctx.ctx, h)
         ctx.step(2)
         assert np.array_equal(ctx.get_kinetic(), want)
+
+
+def test_captured_step_can_be_replayed(kin):
+    # a step captured into a graph advances the state on every replay, between
+    # and after steps that were not captured
+    import torch
+    w = problem((12, 10), (2, 3), 2, 3)
+    st = torch.cuda.Stream()
+    with kin.Context.from_workload(w, stream=st.cuda_stream) as ctx:
+        ctx.set_state(np.ascontiguousarray(w.W0.reshape(-1)))
+        ctx.step(6)
+        want = ctx.get_kinetic()
+        ctx.set_state(np.ascontiguousarray(w.W0.reshape(-1)))
+        ctx.step(1)
+        ctx.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            ctx.step(1)
+        with torch.cuda.stream(st):
+            g.replay()
+            g.replay()
+        ctx.step(1)
+        with torch.cuda.stream(st):
+            g.replay()
+        ctx.step(1)
+        assert np.array_equal(ctx.get_kinetic(), want)
