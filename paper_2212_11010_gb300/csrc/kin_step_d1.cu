@@ -201,6 +201,10 @@ MultiKernel multi_kernel_d1(int degree, int system, int prec, int n, int B)
     const int npop = 2 * nvars(1, system), np = degree + 1, nblk = n / B;
     const long long values = (long long)n * np * npop;
     if (values > (prec == 1 ? 65536 : 16384)) return k;
+    // (FP64 lines of up to 20 nodes: at 16 to 20 a step of 16384 values takes
+    // 10.3 to 12.2 us against 10.7 to 12.8 of one launch per step, and the gain
+    // falls with the chain of a line)
+    if (prec != 1 && B * np > 20) return k;
     k.blocks = values <= (prec == 1 ? 3072 : 1536) ? 1 : 8;
     const int per = (nblk + k.blocks - 1) / k.blocks;
     k.smem = (size_t)(prec == 1 ? 4 : 8) * npop * ((size_t)4 * per + (size_t)per * B * np);
