@@ -233,6 +233,14 @@ static void choose_block(const kin_ctx* c, int B[3])
         bool fits = true;
         for (int a = 0; a < 3; ++a)
             if (c->L[a] % shapes[k][a]) fits = false;
+        // FP64, 2D, p = 3: two waves of the fixed 8 x 4 tiles or the smaller tiles
+        // of the generic kernel -- 10 steps, 8 x 4 against 4 x 4: 16 to 64 tiles
+        // 461 and 308 us, 192 tiles 686 and 629, 384 tiles 1004 and 1112
+        if (c->dim == 2 && c->esize == 8 && c->degree == 3 &&
+            c->n[0] / shapes[k][0] * (c->n[1] / shapes[k][1]) < 2 * 152) {
+            shrink_block(c, B);
+            return;
+        }
         if (fits) {
             for (int a = 0; a < 3; ++a) B[a] = shapes[k][a];
             return;
@@ -595,6 +603,18 @@ static SxArgs sx_args(const kin_ctx* c)
     return S;
 }
 
+// Whether the split 2D sweep is faster than the one-kernel form.  It shortens
+// the chain of every iterate and adds a pass over all cells; at p = 1 a cell
+// solve is short, and with full warps and enough of them per SM the chains of
+// the one-kernel form overlap.  8 steps, p = 1, subdomains of 32^2 cells, one
+// kernel -> split: K = 2 9 subdomains 522 -> 409 us, 30 594 -> 602, 64 686 -> 797;
+// K = 3 30 841 -> 718, 64 949 -> 897.  (p = 2: 1195 -> 793 at 64, K = 2.)
+static bool split_pays(const kin_ctx* c)
+{
+    if (c->degree > 1 || std::min(c->L[0], c->L[1]) <= 16) return true;
+    return 3LL * c->m * c->tiles[0] * c->tiles[1] <= 152LL * std::max(1, 5 * c->iters - 9);
+}
+
 // One step S(dt) for a d + 1 velocity set: K sweeps, then the relaxation.
 // Iterate 1 reads its interface inflow from f^n directly; with K = 1 the
 // sweep writes f^{n+1} in place, so a trace pass copies iterate 0 first.
@@ -898,7 +918,7 @@ kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, 
         if (e == cudaSuccess) {
             e = sx_sweep_plan(sx_args(c), c->precision == KIN_FP32, &c->sx_plan);
             // (the records are an option: without room for them the one-kernel sweep runs)
-            if (e == cudaSuccess && c->dim == 2 && c->precision == KIN_FP32 &&
+            if (e == cudaSuccess && c->dim == 2 && c->precision == KIN_FP32 && split_pays(c) &&
                 dev_alloc(c, sx_split_bytes(sx_args(c)), &c->sxz) == KIN_OK)
                 e = sx_split_plan(sx_args(c), &c->sx_plan);
             c->err.clear();

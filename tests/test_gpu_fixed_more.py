@@ -23,7 +23,7 @@ def kin():
     return kin
 
 
-# (dim, degree, precision, system, block of the default choice, cells per subdomain)
+# (dim, degree, precision, system, block (None: the default choice), cells per subdomain)
 SHAPES = [
     (2, 1, "f32", "euler", (8, 8, 1), 8), (2, 1, "f64", "euler", (8, 8, 1), 8), (2, 3, "f64", "euler", (8, 4, 1), 8),
     (3, 2, "f32", "euler", (4, 2, 2), 4), (3, 3, "f32", "euler", (2, 2, 2), 4),
@@ -60,7 +60,7 @@ def test_matches_oracle(kin, shape, inflow):
     P = oracle.Problem(**w.oracle_kwargs())
     fo = oracle.init(P, w.W0)
     oracle.step(P, fo, 3)
-    with kin.Context.from_workload(w) as ctx:
+    with kin.Context.from_workload(w, **({"block": block} if block else {})) as ctx:
         ctx.set_state(np.ascontiguousarray(w.W0.reshape(-1)))
         ctx.step(3)
         f = ctx.get_kinetic()
