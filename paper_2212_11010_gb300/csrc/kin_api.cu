@@ -471,7 +471,7 @@ static cudaError_t configure_launch(kin_ctx* c)
     if (c->dim == 1 && c->want_stages == 0 && c->want_threads == 0 && c->debug_flags == 0) {
         const MultiKernel mk = multi_kernel_d1(c->degree, c->system, c->precision, c->n[0], c->B[0]);
         if (mk.fn) {
-            e = cudaFuncSetAttribute(mk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mk.smem);
+            e = allow_dynamic_smem(mk.fn);
             c->multi = mk.fn;
             c->multi_smem = mk.smem;
             c->multi_blocks = mk.blocks;

@@ -11,6 +11,17 @@
 
 namespace kin {
 
+cudaError_t allow_dynamic_smem(const void* fn)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+}
+
 // ---------------------------------------------------------------------------
 // Preprocessing (Sec. 3.2: done once, before the time loop), all in FP64 on
 // the device, one thread per (axis, sign).
