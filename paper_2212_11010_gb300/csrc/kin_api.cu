@@ -453,9 +453,7 @@ static cudaError_t configure_launch(kin_ctx* c)
         if (c->stages * tile + tin > 227 * 1024) c->stages = 1;
         c->smem = (int)(c->stages * tile + tin);
     }
-    cudaError_t e = cudaSuccess;
-    if (c->smem > 48 * 1024)
-        e = cudaFuncSetAttribute((const void*)c->kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem);
+    cudaError_t e = allow_dynamic_smem((const void*)c->kfn, (size_t)c->smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void*)c->kfn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int dev = 0, nsm = 1, occ = 1;
@@ -471,7 +469,7 @@ static cudaError_t configure_launch(kin_ctx* c)
     if (c->dim == 1 && c->want_stages == 0 && c->want_threads == 0 && c->debug_flags == 0) {
         const MultiKernel mk = multi_kernel_d1(c->degree, c->system, c->precision, c->n[0], c->B[0]);
         if (mk.fn) {
-            e = allow_dynamic_smem(mk.fn);
+            e = allow_dynamic_smem(mk.fn, mk.smem);
             c->multi = mk.fn;
             c->multi_smem = mk.smem;
             c->multi_blocks = mk.blocks;

@@ -11,7 +11,7 @@
 
 namespace kin {
 
-cudaError_t allow_dynamic_smem(const void* fn)
+cudaError_t allow_dynamic_smem(const void* fn, size_t need)
 {
     int dev = 0, most = 0;
     cudaFuncAttributes at;
@@ -19,7 +19,9 @@ cudaError_t allow_dynamic_smem(const void* fn)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+    most -= (int)at.sharedSizeBytes;
+    if (need > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // ---------------------------------------------------------------------------

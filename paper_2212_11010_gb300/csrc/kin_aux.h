@@ -15,8 +15,9 @@ struct Inst;
 // Lets a kernel be launched with all the dynamic shared memory that a block can
 // have beside its static one.  The limit belongs to the function, and contexts
 // of different sizes share functions: set to one context's own size it would
-// stop the launches of a larger one created before.
-cudaError_t allow_dynamic_smem(const void* fn);
+// stop the launches of a larger one created before.  cudaErrorInvalidValue
+// when 'need' bytes are more than that.
+cudaError_t allow_dynamic_smem(const void* fn, size_t need);
 
 // Constants of the relaxation in both precisions, computed once on the host:
 // one FP64 operation of a warp occupies the SM's FP64 units for 16 cycles, and

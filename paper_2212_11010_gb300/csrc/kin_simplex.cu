@@ -1631,7 +1631,7 @@ cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
                        : wave_pick<double>(a.dim, a.degree, plan->threads);
     // (the brick kernel's shared memory stays below 48 KB)
     e = plan->brick ? cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)
-                                : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem);
+                    : allow_dynamic_smem(fn, plan->smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, plan->threads, plan->smem);

@@ -27,10 +27,19 @@ def line(n, degree, prec):
     return workloads.advection1d(seed=n, n=n, tiles=4, degree=degree, dt=2.4 / n, precision=prec), {}
 
 
-# (larger, smaller): several steps per launch in 1D, one block or eight
+def plane(n, tiles, degree, block, prec="f32"):
+    w = workloads.vortex2d(seed=n, n=n, degree=degree, tiles=tiles, dt_mult=4.0)
+    return workloads.with_(w, precision=prec), dict(block=block) if block else {}
+
+
+# (larger, smaller): several steps per launch in 1D, one block or eight; the
+# generic kernel with tiles of 50 to 220 KB
 PAIRS = {
     "1d-f32": (line(8192, 3, "f32"), line(256, 3, "f32")),
     "1d-f64": (line(4096, 1, "f64"), line(64, 1, "f64")),
+    "2d-p1": (plane(116, 4, 1, (29, 29)), plane(68, 4, 1, (17, 17))),
+    "2d-p2": (plane(39, 3, 2, (13, 13)), plane(33, 3, 2, (11, 11))),
+    "2d-p3-f64": (plane(28, 4, 3, (7, 7), "f64"), plane(20, 4, 3, (5, 5), "f64")),
 }
 
 
@@ -73,3 +82,35 @@ def test_larger_context_survives_a_smaller_one(kin, name):
             batch.sync()
         assert np.array_equal(a.get_kinetic(), alone[0])
         assert np.array_equal(b.get_kinetic(), alone[1])
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_wavefront_sweeps_of_two_sizes(kin, dim, prec):
+    # one kernel instance for up to 256 columns per subdomain (3D: degree 2)
+    if dim == 2:
+        ws = [workloads.vortex2d(seed=n, n=n, degree=2, tiles=1, dt_mult=4.0, velset=1) for n in (200, 12)]
+        if prec == "f32":           # without room for its records: the sweep in one kernel
+            with kin.Context.from_workload(ws[0]) as ctx:
+                need = ctx.info.device_bytes - 256
+    else:
+        ws = [workloads.densitywave3d(seed=n, n=n, degree=2, tiles=1, dt_mult=4.0, velset=1) for n in (12, 4)]
+    ws = [workloads.with_(w, precision=prec) for w in ws]
+    kw = [{}, {}]
+    if dim == 2 and prec == "f32":
+        kw[0] = dict(mem_budget=need)
+    alone = []
+    for w, k in zip(ws, kw):
+        with kin.Context.from_workload(w, **k) as ctx:
+            alone.append(run(ctx, w, 2))
+    with kin.Context.from_workload(ws[0], **kw[0]) as a, kin.Context.from_workload(ws[1], **kw[1]) as b:
+        assert np.array_equal(run(b, ws[1], 2), alone[1])
+        assert np.array_equal(run(a, ws[0], 2), alone[0])
+
+
+def test_a_block_beyond_shared_memory_is_refused(kin):
+    # a tile of 230,400 bytes fits 227 KB, its inflow traces beside it do not
+    w, k = plane(30, 1, 1, (30, 30))
+    with pytest.raises(kin.KinError) as e:
+        kin.Context.from_workload(w, **k)
+    assert e.value.status == kin.KIN_ECUDA
