@@ -76,7 +76,7 @@ struct kin_ctx {
     void* sxz = nullptr;              // split sweep (2D, FP32): records; NULL when they did not fit the budget
     int sxz_parity = 0;
     bool sxz_ready = false;           // the records are those of f
-    bool sxz_captured = false;        // a step was captured into a graph, which may be replayed at any time
+    bool sxz_captured = false;        // work that writes f was captured into a graph (note_capture)
     int sx_stride = 0;
     // tetrahedral meshes
     bool tet = false;
@@ -613,6 +613,18 @@ static bool split_pays(const kin_ctx* c)
     return 3LL * c->m * c->tiles[0] * c->tiles[1] <= 152LL * std::max(1, 5 * c->iters - 9);
 }
 
+// To be called before work that writes f is put on stream st.  Work captured
+// into a graph, a step or a new state, may be replayed at any time without this
+// context knowing: from the first on, every step computes its own records.
+static cudaError_t note_capture(kin_ctx* c, cudaStream_t st)
+{
+    if (!c->sxz || c->sxz_captured || !st || st == cudaStreamLegacy) return cudaSuccess;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    if (e == cudaSuccess) c->sxz_captured = cs != cudaStreamCaptureStatusNone;
+    return e;
+}
+
 // One step S(dt) for a d + 1 velocity set: K sweeps, then the relaxation.
 // Iterate 1 reads its interface inflow from f^n directly; with K = 1 the
 // sweep writes f^{n+1} in place, so a trace pass copies iterate 0 first.
@@ -625,13 +637,7 @@ static kin_status sx_step(kin_ctx* c)
         KIN_CUDA(c, sx_launch_trace0(S, prec, c->stream));
     }
     if (c->sxz) {
-        // a replayed graph advances f without this context knowing: from the
-        // first captured step on, every step computes its own records
-        if (c->stream && !c->sxz_captured) {
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            KIN_CUDA(c, cudaStreamIsCapturing(c->stream, &cs));
-            c->sxz_captured = cs != cudaStreamCaptureStatusNone;
-        }
+        KIN_CUDA(c, note_capture(c, c->stream));
         if (c->sxz_captured) c->sxz_ready = false;
         KIN_CUDA(c, sx_split_step(S, c->sx_hrec.data(), c->sx_stride, c->sx_plan, c->sxz, c->sxz_parity, c->sxz_ready,
                                   c->iters, c->sxtr, c->stream));
@@ -1464,6 +1470,7 @@ kin_status kin_set_state(kin_ctx* c, const double* W, size_t n_values, int on_de
     if (c->tet) {
         KIN_CUDA(c, tet_launch_init(tet_args(c), src, c->precision == KIN_FP32, c->stream));
     } else if (c->simplex) {
+        KIN_CUDA(c, note_capture(c, c->stream));
         KIN_CUDA(c, sx_launch_init(sx_args(c), src, c->precision == KIN_FP32, c->stream));
         c->sxz_ready = false;
     } else {
@@ -1489,6 +1496,7 @@ kin_status kin_set_kinetic(kin_ctx* c, const void* f, size_t n_values, int on_de
     if (!f) return fail(c, KIN_EINVAL, "f is NULL");
     if (n_values != (size_t)c->npop * c->nodes)
         return fail(c, KIN_EINVAL, "expected %zu values, got %zu", (size_t)c->npop * c->nodes, n_values);
+    KIN_CUDA(c, note_capture(c, c->stream));
     KIN_CUDA(c, cudaMemcpyAsync(c->f, f, n_values * c->esize,
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
     c->sxz_ready = false;
@@ -1514,6 +1522,7 @@ kin_status kin_set_kinetic_async(kin_ctx* c, const void* f, size_t n_values, voi
     if (n_values != (size_t)c->npop * c->nodes)
         return fail(c, KIN_EINVAL, "expected %zu values, got %zu", (size_t)c->npop * c->nodes, n_values);
     cudaStream_t s = stream ? (cudaStream_t)stream : c->stream;
+    KIN_CUDA(c, note_capture(c, s));
     KIN_CUDA(c, cudaMemcpyAsync(c->f, f, n_values * c->esize, cudaMemcpyHostToDevice, s));
     // the interface summaries of the new f are computed by the next step
     // (kin_step, kin_batch_step) or diagnostic that needs them
