@@ -1311,7 +1311,7 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
                 int cells = C;                           // cells of the open chunk (C: none is open)
                 for (int q = V.bounds[l]; q < V.bounds[l + 1]; ++q) {
                     const int cc = ord[q];
-                    int nh = 0, out = 0;
+                    int nh = 0;
                     for (int a = 0; a < 4; ++a) nh += inflow(k, cc, a) && ((iface[cc] >> a) & 1);
                     if (C == 0 ? q == V.bounds[l] : cells == C || (int)K.hcell.size() - K.hstart.back() + nh > C) {
                         K.bounds.push_back(q);
@@ -1322,10 +1322,7 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
                     for (int a = 0; a < 4; ++a) {
                         const int R0 = (int)mesh->nbr[(size_t)cc * 4 + a];
                         const bool itf = (iface[cc] >> a) & 1;
-                        if (!inflow(k, cc, a)) {
-                            if (itf) out = kTetOutFace;
-                            continue;
-                        }
+                        if (!inflow(k, cc, a)) continue;
                         int src = R0;
                         if (C > 0 && itf) {
                             src = (int)K.hcell.size() - K.hstart.back();
@@ -1338,13 +1335,15 @@ kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, doubl
                             wd |= (fnodes[(size_t)cc * 12 + a * 3 + jj] & 3) << (5 - 2 * jj);
                         fr[(size_t)q * 4 + a] = wd;
                     }
-                    if (C > 0) ord[q] |= out;
                 }
             }
         }
         K.start.push_back((int)K.bounds.size());
         K.bounds.push_back(n);
         K.hstart.push_back((int)K.hcell.size());
+        // what others read is decided by the readers: the two cells of a face may
+        // disagree about it (a cell may name a neighbour that does not name it)
+        for (int cc : K.hcell) ord[rk[cc]] |= kTetOutFace;
     });
     if (!ran) {
         delete c;
