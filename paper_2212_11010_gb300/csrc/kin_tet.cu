@@ -127,8 +127,41 @@ __global__ void tet_setup_kernel(TetSetupArgs A)
         for (int j = 0; j < 4; ++j) rec[i * 4 + j] = M[i][4 + j] * (vol / 20.0);
     for (int a = 0; a < 4; ++a) rec[16 + a] = cin[a] / (vol / 20.0);
     if (A.c32) {
+        // Rounded entry by entry, B acts on sums whose terms nearly cancel, and on a
+        // mesh of congruent cells every cell and step has the same error: it adds
+        // up (Maxwell, D3Q6, 8 steps: 2.5e-6 of the norm, 6e-7 with an exact B).
+        // What counts is its effect on fields that are constant over the nodes,
+        // B q with q_j = 5 + 4 (sum of the factors of the faces at node j) (the
+        // rows of B q = 1): in each row the four entries are rounded up or down so
+        // that the sum of their errors times q is smallest (6.5e-7).
         float* r32 = A.c32 + ((size_t)k * A.ncells + pos) * kTetRec;
-        for (int q = 0; q < kTetRec; ++q) r32[q] = (float)rec[q];
+        double q[4] = {5.0, 5.0, 5.0, 5.0};
+        for (int a = 0; a < 4; ++a) {
+            r32[16 + a] = (float)rec[16 + a];
+            for (int j = 0; j < 4; ++j)
+                if (j != a) q[j] += 4.0 * r32[16 + a];
+        }
+        for (int i = 0; i < 4; ++i) {
+            float lo[4], hi[4];
+            double off = 0.0, up[4], least = 0.0;
+            for (int j = 0; j < 4; ++j) {
+                lo[j] = __double2float_rd(rec[i * 4 + j]);
+                hi[j] = __double2float_ru(rec[i * 4 + j]);
+                off += ((double)lo[j] - rec[i * 4 + j]) * q[j];
+                up[j] = ((double)hi[j] - (double)lo[j]) * q[j];
+            }
+            int best = 0;
+            for (int mask = 0; mask < 16; ++mask) {
+                double d = off;
+                for (int j = 0; j < 4; ++j)
+                    if ((mask >> j) & 1) d += up[j];
+                if (mask == 0 || fabs(d) < least) {
+                    least = fabs(d);
+                    best = mask;
+                }
+            }
+            for (int j = 0; j < 4; ++j) r32[i * 4 + j] = (best >> j) & 1 ? hi[j] : lo[j];
+        }
     }
 }
 
@@ -484,19 +517,20 @@ __global__ void __launch_bounds__(kTetRingThreads)
 #pragma unroll
             for (int v = 0; v < VPT; ++v) {
                 if (MV % VPT != 0 && vg * VPT + v >= MV) break;
-                T x[4];
+                T x[4], d[4];
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    T acc = rec[b * 4] * rhs[v][0];
+                    d[b] = rec[b * 4] * rhs[v][0];
 #pragma unroll
-                    for (int j = 1; j < 4; ++j) acc = fma(rec[b * 4 + j], rhs[v][j], acc);
-                    x[b] = acc + u[v][0];
+                    for (int j = 1; j < 4; ++j) d[b] = fma(rec[b * 4 + j], rhs[v][j], d[b]);
+                    x[b] = d[b] + u[v][0];
                 }
                 store4(ring + (slot * MV + vg * VPT + v) * 4, x);
                 if (vg * VPT + v >= mvb) continue;
                 if (final) {
+                    // 2 x - f^n without the rounding of x
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) x[b] = fma(T(2), x[b], -u[v][b]);
+                    for (int b = 0; b < 4; ++b) x[b] = fma(T(2), d[b] + (u[v][0] - u[v][b]), u[v][b]);
                     store4(fp + (vg * VPT + v) * nodes + c4, x);
                 } else if (send) {
                     store4(cur + pop + (vg * VPT + v) * nodes + c4, x);
