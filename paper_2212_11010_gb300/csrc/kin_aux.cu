@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ 
             using V = std::remove_cv_t<std::remove_reference_t<decltype(w[0])>>;
             const InitK<V>& K = init_k<V>(A);
             V Q[D][M];
-            init_flux<D, SYS, V>(K, w, Q);
+            float worst = init_flux<D, SYS, V>(K, w, Q);
 #pragma unroll
             for (int v = 0; v < M; ++v) {
                 V base;
@@ -236,10 +236,12 @@ __global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ 
                     // (Maxwell: Q^a has no component along E_a and H_a)
                     const bool z = SYS == kMaxwell && (v == a || v == 3 + a);
                     const V half = Q[a][v] * K.inv2l;
-                    init_put(f[(long long)((2 * a) * M + v) * nodes + i], z ? base : base + half);
-                    init_put(f[(long long)((2 * a + 1) * M + v) * nodes + i], z ? base : base - half);
+                    const float mag = init_mag(base);
+                    init_put<SYS>(f[(long long)((2 * a) * M + v) * nodes + i], z ? base : base + half, mag, worst);
+                    init_put<SYS>(f[(long long)((2 * a + 1) * M + v) * nodes + i], z ? base : base - half, mag, worst);
                 }
             }
+            return worst >= 0.0f;
         });
     }
 }

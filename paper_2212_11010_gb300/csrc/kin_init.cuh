@@ -7,17 +7,25 @@
 // divisions.  Before, 128^3 cells of 3D Euler (p = 1, 2.7 GB) took 11.2 ms, 4%
 // of the copy rate; now 0.6 ms (67%).  An FP64 state keeps its FP64
 // operations, with one reciprocal per node instead of a division per use
-// (48^3 cells of Maxwell: 0.64 -> 0.08 ms).  For an FP32 state the Maxwellians are therefore evaluated on
-// unevaluated FP32 pairs (Dekker, "A floating-point technique for extending
-// the available precision", 1971; 47 bits), whose rounding to FP32 differs
-// from that of the FP64 value only where the latter lies within 2^-22 of an
-// ulp from a tie.  The double is split into its pair with integer
-// instructions, so a node issues no FP64 instruction at all.  Values outside
-// the range in which no partial result can leave the FP32 exponent range
-// (init_fast) take the FP64 evaluation.
+// (48^3 cells of Maxwell: 0.64 -> 0.08 ms).  For an FP32 state the Maxwellians
+// are therefore evaluated on unevaluated FP32 pairs (Dekker, "A floating-point
+// technique for extending the available precision", 1971; 47 bits).  The double
+// is split into its pair with integer instructions, so a node issues no FP64
+// instruction at all.
+//   What a pair loses against FP64 counts where values cancel: the pressure is a
+// small difference at high Mach numbers, and W/(2d) -+ Q/(2 lambda) changes
+// sign.  Each node checks that (init_flux, init_put), and one where a difference
+// is smaller than 2^-5 (pressure) or 2^-6 (2^-12 for the linear systems) of its terms, or
+// whose values leave the range in which no partial result can leave the FP32 exponent
+// range (init_fast), is evaluated again in FP64.  So every value is
+// off by less than 2^-32 of itself before its rounding to FP32: an input is cut
+// to 2^-47, a product or sum adds at most 2^-45, at most eight of them follow
+// one another, and the two differences lose 5 and 6 bits.
 #pragma once
 
 #include <math.h>
+
+#include <type_traits>
 
 #include "kin_device.cuh"
 
@@ -99,10 +107,16 @@ template <typename V> __device__ __forceinline__ const InitK<V>& init_k(const In
 template <> __device__ __forceinline__ const InitK<double>& init_k<double>(const InitArgs& A) { return A.kd; }
 template <> __device__ __forceinline__ const InitK<F2>& init_k<F2>(const InitArgs& A) { return A.kf; }
 
-// Q^a(W) for every axis: Euler, advection, or Maxwell (3D; Sec. 6.1.1).
+// Magnitude of a value, for the checks of the pair arithmetic.
+__device__ __forceinline__ float init_mag(F2 x) { return fabsf(x.h); }
+__device__ __forceinline__ float init_mag(double) { return 0.0f; }
+
+// Q^a(W) for every axis: Euler, advection, or Maxwell (3D; Sec. 6.1.1).  Negative
+// when the pressure is less than 2^-5 of (gamma - 1) E (pairs), else zero.
 template <int D, int SYS, typename V>
-__device__ __forceinline__ void init_flux(const InitK<V>& K, const V* W, V (*Q)[nvars(D, SYS)])
+__device__ __forceinline__ float init_flux(const InitK<V>& K, const V* W, V (*Q)[nvars(D, SYS)])
 {
+    float worst = 0.0f;
     if constexpr (SYS == kAdvection) {
 #pragma unroll
         for (int a = 0; a < D; ++a) Q[a][0] = K.adv[a] * W[0];
@@ -115,7 +129,8 @@ __device__ __forceinline__ void init_flux(const InitK<V>& K, const V* W, V (*Q)[
         V ke = W[1] * W[1];
 #pragma unroll
         for (int b = 1; b < D; ++b) ke = ke + W[1 + b] * W[1 + b];
-        const V pr = K.gm1 * (W[1 + D] - init_const<V>(0.5) * (ke * inv));
+        const V in = W[1 + D] - init_const<V>(0.5) * (ke * inv), pr = K.gm1 * in;
+        if constexpr (std::is_same<V, F2>::value) worst = fminf(0.0f, fmaf(-0.03125f, W[1 + D].h, in.h));
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             const V ua = W[1 + a] * inv;
@@ -128,13 +143,14 @@ __device__ __forceinline__ void init_flux(const InitK<V>& K, const V* W, V (*Q)[
             Q[a][1 + D] = (W[1 + D] + pr) * ua;
         }
     }
+    return worst;
 }
 
 // Whether the pair arithmetic may be used on W: every value zero or in
 // [2^-75, 2^100) when nothing but constants multiplies it, in
-// [2^-75, 2^24) with rho >= 2^-12 for Euler, so that the largest product
-// ((E + p) u, below 2^108 with gamma - 1 < 2^8) stays finite.  NaN and
-// infinities fail the test.  (lambda and the other constants are checked on
+// [2^-48, 2^24) with rho >= 2^-12 for Euler, so that the largest product
+// ((E + p) u, below 2^108 with gamma - 1 < 2^8) stays finite and the smallest
+// (m^2 / rho, 2^-120) is not zero.  NaN and infinities fail the test.  (lambda and the other constants are checked on
 // the host, init_fast_model.)
 template <int M, int SYS>
 __device__ __forceinline__ bool init_fast(const unsigned (&hi)[M], const unsigned (&lo)[M])
@@ -143,8 +159,8 @@ __device__ __forceinline__ bool init_fast(const unsigned (&hi)[M], const unsigne
 #pragma unroll
     for (int v = 0; v < M; ++v) {
         const unsigned a = hi[v] & 0x7fffffffu;
-        const unsigned top = SYS == kEuler ? 1023u + 24u : 1023u + 100u;
-        ok = ok && ((a | lo[v]) == 0 || (a >= ((1023u - 75u) << 20) && a < (top << 20)));
+        const unsigned top = SYS == kEuler ? 1023u + 24u : 1023u + 100u, low = SYS == kEuler ? 1023u - 48u : 1023u - 75u;
+        ok = ok && ((a | lo[v]) == 0 || (a >= (low << 20) && a < (top << 20)));
     }
     if (SYS == kEuler) ok = ok && hi[0] >= ((1023u - 12u) << 20) && hi[0] < 0x7ff00000u;
     return ok;
@@ -158,35 +174,45 @@ inline int init_fast_model(double lambda, double gamma, const double* adv)
 }
 
 // emit(W) with the node's m values, as pairs where the state is FP32 and the
-// values allow it, else as doubles.
+// values allow it; as doubles else, and where emit on pairs returns false (a
+// value that it stored has lost too much and is stored again).
 template <int D, int SYS, typename T, typename E>
 __device__ __forceinline__ void init_node(const double* __restrict__ Wd, long long nodes, long long i, int fast,
                                           const E& emit)
 {
     constexpr int M = nvars(D, SYS);
     double w[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) w[v] = __ldg(Wd + (long long)v * nodes + i);
     if constexpr (sizeof(T) == 4) {
         unsigned hi[M], lo[M];
 #pragma unroll
         for (int v = 0; v < M; ++v) {
-            hi[v] = (unsigned)__double2hiint(w[v]);
-            lo[v] = (unsigned)__double2loint(w[v]);
+            const double x = __ldg(Wd + (long long)v * nodes + i);
+            hi[v] = (unsigned)__double2hiint(x);
+            lo[v] = (unsigned)__double2loint(x);
         }
         if (fast && init_fast<M, SYS>(hi, lo)) {
             F2 W[M];
 #pragma unroll
             for (int v = 0; v < M; ++v) W[v] = f2_of_bits(hi[v], lo[v]);
-            emit(W);
-            return;
+            if (emit(W)) return;
         }
     }
+    // (read again: held over the pairs they cost registers on every node)
+#pragma unroll
+    for (int v = 0; v < M; ++v) w[v] = *(const volatile double*)(Wd + (long long)v * nodes + i);
     emit(w);
 }
 
-__device__ __forceinline__ void init_put(float& f, F2 x) { f = x.h; }
-template <typename T>
-__device__ __forceinline__ void init_put(T& f, double x) { f = (T)x; }
+// Stores x, the sum of terms of magnitude mag; worst becomes negative when x has
+// lost more than 6 bits (12 for the linear systems) to cancellation.
+template <int SYS>
+__device__ __forceinline__ void init_put(float& f, F2 x, float mag, float& worst)
+{
+    constexpr float part = SYS == kEuler ? 0.015625f : 0.000244140625f;
+    f = x.h;
+    worst = fminf(worst, fmaf(-part, mag, fabsf(x.h)));
+}
+template <int SYS, typename T>
+__device__ __forceinline__ void init_put(T& f, double x, float, float&) { f = (T)x; }
 
 }  // namespace kin

@@ -1503,7 +1503,7 @@ __global__ void __launch_bounds__(256) sx_init_kernel(const __grid_constant__ Sx
         init_node<D, SYS, T>(Wd, nodes, i, S.A.fast, [&](const auto& W) {
             using V = std::remove_cv_t<std::remove_reference_t<decltype(W[0])>>;
             V Q[D][M];
-            init_flux<D, SYS, V>(init_k<V>(S.A), W, Q);
+            float worst = init_flux<D, SYS, V>(init_k<V>(S.A), W, Q);
 #pragma unroll
             for (int kk = 0; kk < NV; ++kk)
 #pragma unroll
@@ -1513,10 +1513,16 @@ __global__ void __launch_bounds__(256) sx_init_kernel(const __grid_constant__ Sx
                         else return S.mf[kk * NV + j];
                     };
                     V mk = mi(0) * W[v];
+                    float mag = init_mag(mk);
 #pragma unroll
-                    for (int a = 0; a < D; ++a) mk = mk + mi(1 + a) * Q[a][v];
-                    init_put(f[(long long)(kk * M + v) * nodes + i], mk);
+                    for (int a = 0; a < D; ++a) {
+                        const V q = mi(1 + a) * Q[a][v];
+                        mk = mk + q;
+                        mag += init_mag(q);
+                    }
+                    init_put<SYS>(f[(long long)(kk * M + v) * nodes + i], mk, mag, worst);
                 }
+            return worst >= 0.0f;
         });
     }
 }

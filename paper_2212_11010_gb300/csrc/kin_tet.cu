@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(256) tet_init_kernel(const __grid_constant__ I
             using V = std::remove_cv_t<std::remove_reference_t<decltype(W[0])>>;
             const InitK<V>& K = init_k<V>(A);
             V Q[3][m];
-            init_flux<3, SYS, V>(K, W, Q);
+            float worst = init_flux<3, SYS, V>(K, W, Q);
 #pragma unroll
             for (int v = 0; v < m; ++v) {
                 if constexpr (VS == 1) {
@@ -741,10 +741,11 @@ __global__ void __launch_bounds__(256) tet_init_kernel(const __grid_constant__ I
                     const V qx = Q[0][v] * il, qy = Q[1][v] * il, qz = Q[2][v] * il;
                     const V a = base + qx, b = base - qx, s = qy + qz, d = qy - qz;
                     // signs (+,+,+), (+,-,-), (-,+,-), (-,-,+)
-                    init_put(f[(long long)(0 * m + v) * nodes + i], a + s);
-                    init_put(f[(long long)(1 * m + v) * nodes + i], a - s);
-                    init_put(f[(long long)(2 * m + v) * nodes + i], b + d);
-                    init_put(f[(long long)(3 * m + v) * nodes + i], b - d);
+                    const float mag = init_mag(base) + init_mag(qx) + init_mag(qy) + init_mag(qz);
+                    init_put<SYS>(f[(long long)(0 * m + v) * nodes + i], a + s, mag, worst);
+                    init_put<SYS>(f[(long long)(1 * m + v) * nodes + i], a - s, mag, worst);
+                    init_put<SYS>(f[(long long)(2 * m + v) * nodes + i], b + d, mag, worst);
+                    init_put<SYS>(f[(long long)(3 * m + v) * nodes + i], b - d, mag, worst);
                 } else {
                     V base;
                     if constexpr (std::is_same<V, double>::value) base = div2d<3>(W[v]);
@@ -752,11 +753,12 @@ __global__ void __launch_bounds__(256) tet_init_kernel(const __grid_constant__ I
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         const V q = Q[a][v] * K.inv2l;
-                        init_put(f[(long long)((2 * a) * m + v) * nodes + i], base + q);
-                        init_put(f[(long long)((2 * a + 1) * m + v) * nodes + i], base - q);
+                        init_put<SYS>(f[(long long)((2 * a) * m + v) * nodes + i], base + q, init_mag(base), worst);
+                        init_put<SYS>(f[(long long)((2 * a + 1) * m + v) * nodes + i], base - q, init_mag(base), worst);
                     }
                 }
             }
+            return worst >= 0.0f;
         });
     }
 }
