@@ -223,9 +223,13 @@ static void shrink_block(const kin_ctx* c, int B[3])
 //   Time: a tile's phases take about 10,000 cycles of latency whatever its
 // size, shared by the tiles resident on an SM, plus their instructions.
 //   290 x 210 cells, p = 1, subdomains of 29 x 35: 130 us per step with the
-// shrunk 1 x 7 blocks, 22 us with 29 x 5.  A block never needs more summary
-// memory than the shrunk one (its thinnest extent is no smaller).
-static void choose_block(const kin_ctx* c, int B[3])
+// shrunk 1 x 7 blocks, 22 us with 29 x 5.  An estimated block never needs more
+// summary memory than the shrunk one (its thinnest extent is no smaller), and of
+// the compiled shapes only 8 x 8 (2D, p = 1, FP32; subdomains of 24, 40 or 56
+// cells) can: half as much again against 12 x 12, at 0.5 to 0.6 times its time
+// (648^2 cells 53.5 against 87.1 us per step, 320^2 15.0 against 26.7).  True is returned
+// for it, and with 'thick' it is left out: for problems whose memory limit it exceeds.
+static bool choose_block(const kin_ctx* c, int B[3], bool thick)
 {
     int shapes[4][3];
     const int ns = fixed_shapes(c->dim, c->degree, c->system, c->precision, shapes);
@@ -239,15 +243,21 @@ static void choose_block(const kin_ctx* c, int B[3])
         if (c->dim == 2 && c->esize == 8 && c->degree == 3 &&
             c->n[0] / shapes[k][0] * (c->n[1] / shapes[k][1]) < 2 * 152) {
             shrink_block(c, B);
-            return;
+            return false;
         }
         if (fits) {
+            bool thin = false;
+            if (c->dim == 2 && c->esize == 4 && c->degree == 1 && shapes[k][0] == 8 && shapes[k][1] == 8) {
+                shrink_block(c, B);
+                thin = std::min(B[0], B[1]) > 8;
+            }
+            if (thin && thick) continue;
             for (int a = 0; a < 3; ++a) B[a] = shapes[k][a];
-            return;
+            return thin;
         }
     }
     shrink_block(c, B);
-    if (c->dim < 2 || c->want_stages == 2) return;      // two tile buffers: the small tiles
+    if (c->dim < 2 || c->want_stages == 2) return false;      // two tile buffers: the small tiles
     int least = B[0];
     for (int a = 1; a < c->dim; ++a) least = std::min(least, B[a]);
     std::vector<int> div[3];
@@ -289,6 +299,7 @@ static void choose_block(const kin_ctx* c, int B[3])
                     for (int a = 0; a < 3; ++a) B[a] = b[a];
                 }
             }
+    return false;
 }
 
 // Bulk copies need every row of a cell block to start on a 16-byte
@@ -732,11 +743,11 @@ static bool each_velocity(int nvel, const F& fn)
     return ok;
 }
 
-extern "C" {
-
-kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, double dt,
-                      const kin_opts* opts, kin_ctx** out)
+// kin_create; *thin: the default block could be thicker, which 'thick' asks for.
+static kin_status create_grid(const kin_mesh* mesh, const kin_model* model, int degree, double dt,
+                              const kin_opts* opts, kin_ctx** out, bool thick, bool* thin)
 {
+    *thin = false;
     if (!out) return fail(nullptr, KIN_EINVAL, "out is NULL");
     *out = nullptr;
     if (!mesh || !model || !opts) return fail(nullptr, KIN_EINVAL, "mesh, model and opts are required");
@@ -953,7 +964,7 @@ kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, 
             c->B[a] = b;
         }
     } else {
-        choose_block(c, c->B);
+        *thin = choose_block(c, c->B, thick);
     }
     for (int a = 0; a < 3; ++a) {
         c->nblk[a] = c->n[a] / c->B[a];
@@ -1049,6 +1060,18 @@ kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, 
     }
     *out = c;
     return KIN_OK;
+}
+
+extern "C" {
+
+kin_status kin_create(const kin_mesh* mesh, const kin_model* model, int degree, double dt,
+                      const kin_opts* opts, kin_ctx** out)
+{
+    bool thin;
+    kin_status st = create_grid(mesh, model, degree, dt, opts, out, false, &thin);
+    if (thin && (st == KIN_EBUDGET || st == KIN_ENOMEM))
+        st = create_grid(mesh, model, degree, dt, opts, out, true, &thin);
+    return st;
 }
 
 kin_status kin_create_tet(const kin_tetmesh* mesh, const kin_model* model, double dt, const kin_opts* opts,
@@ -2348,7 +2371,8 @@ extern "C" kin_status kin_step_noalloc(const kin_mesh* mesh, const kin_model* mo
         c.cells *= c.n[a];
     }
     c.nodes = c.cells * c.NN;
-    if (opts->block[0] || opts->block[1] || opts->block[2]) {
+    const bool user_block = opts->block[0] || opts->block[1] || opts->block[2];
+    if (user_block) {
         for (int a = 0; a < 3; ++a) {
             int b = a < c.dim ? opts->block[a] : 1;
             if (b < 1 || c.L[a] % b) {
@@ -2357,38 +2381,36 @@ extern "C" kin_status kin_step_noalloc(const kin_mesh* mesh, const kin_model* mo
             }
             c.B[a] = b;
         }
-    } else {
-        choose_block(&c, c.B);
-    }
-    for (int a = 0; a < 3; ++a) {
-        c.nblk[a] = c.n[a] / c.B[a];
-        c.nb[a] = c.L[a] / c.B[a];
-    }
-    const size_t smem = block_smem(&c, c.B);
-    if (smem > 227 * 1024) {
-        noalloc_msg(errbuf, errlen, "cell block needs %zu bytes of shared memory (> 227 KB)", smem);
-        return KIN_EINVAL;
     }
     c.kfn = pick_kernel(c.dim, degree, c.system, c.precision);
-    size_t tn = 1;
-    for (int a = 1; a < c.dim; ++a) tn *= c.NP;
-    size_t stride = 0, rstride = 0;
-    for (int a = 0; a < c.dim; ++a) {
-        stride = std::max(stride, (size_t)c.nblk[a] * (c.cells / c.n[a]) * tn);
-        rstride = std::max(rstride, (size_t)c.tiles[a] * (c.cells / c.n[a]) * tn);
-    }
-    c.sig_stride = stride;
-    c.raw_stride = rstride;
-
     // scratch layout: c64 | c32 | gll | error word | sig0 | raw0 | sig1 | raw1
     const size_t off_c64 = 0;
     const size_t off_c32 = align256(off_c64 + sizeof(double) * 6 * kCoefStride);
     const size_t off_gll = align256(off_c32 + sizeof(float) * 6 * kCoefStride);
     const size_t off_err = align256(off_gll + sizeof(double) * 2 * kMaxNP);
     const size_t off_sum = align256(off_err + sizeof(int) * 4);
-    const size_t sbytes = align256(stride * c.npop * c.esize);
-    const size_t rbytes = align256(rstride * c.npop * c.esize);
-    const size_t need = off_sum + 2 * sbytes + 2 * rbytes;
+    size_t tn = 1, sbytes = 0, rbytes = 0, need = 0;
+    for (int a = 1; a < c.dim; ++a) tn *= c.NP;
+    for (bool thick = false;; thick = true) {
+        const bool thin = !user_block && choose_block(&c, c.B, thick);
+        c.sig_stride = c.raw_stride = 0;
+        for (int a = 0; a < 3; ++a) {
+            c.nblk[a] = c.n[a] / c.B[a];
+            c.nb[a] = c.L[a] / c.B[a];
+            if (a >= c.dim) continue;
+            c.sig_stride = std::max(c.sig_stride, (size_t)c.nblk[a] * (c.cells / c.n[a]) * tn);
+            c.raw_stride = std::max(c.raw_stride, (size_t)c.tiles[a] * (c.cells / c.n[a]) * tn);
+        }
+        const size_t smem = block_smem(&c, c.B);
+        if (smem > 227 * 1024) {
+            noalloc_msg(errbuf, errlen, "cell block needs %zu bytes of shared memory (> 227 KB)", smem);
+            return KIN_EINVAL;
+        }
+        sbytes = align256(c.sig_stride * c.npop * c.esize);
+        rbytes = align256(c.raw_stride * c.npop * c.esize);
+        need = off_sum + 2 * sbytes + 2 * rbytes;
+        if (need <= kNoallocScratchBytes || !thin) break;
+    }
     if (need > kNoallocScratchBytes) {
         noalloc_msg(errbuf, errlen,
                     "problem needs %zu bytes of scratch; kin_step_noalloc is limited to %zu bytes "
