@@ -613,15 +613,33 @@ static SxArgs sx_args(const kin_ctx* c)
 }
 
 // Whether the split 2D sweep is faster than the one-kernel form.  It shortens
-// the chain of every iterate and adds a pass over all cells; at p = 1 a cell
-// solve is short, and with full warps and enough of them per SM the chains of
-// the one-kernel form overlap.  8 steps, p = 1, subdomains of 32^2 cells, one
-// kernel -> split: K = 2 9 subdomains 522 -> 409 us, 30 594 -> 602, 64 686 -> 797;
-// K = 3 30 841 -> 718, 64 949 -> 897.  (p = 2: 1195 -> 793 at 64, K = 2.)
+// the chain of every iterate and adds a pass over all cells per step, so it pays
+// the more iterates there are, the longer a cell solve is and the fewer columns
+// (lanes) share the SMs: with full warps the chains of the one-kernel form overlap.
+// Time of one kernel / split, square subdomains of 8 to 128 cells, up to 2048^2
+// cells (p = 3: 1024^2):
+//   p = 1, K = 1: 1.06 to 1.26 up to 256 columns, 0.47 to 0.85 from 512 on and 0.8 to
+//          0.95 with 8 cells; K = 2: 1.1 to 1.5 up to 512 columns, 0.67 to 0.98 from 1024
+//          on, with 8 cells 1.0 to 1.4; K = 3: 1.1 to 1.7 up to 1280 columns, 0.92 to 1.02
+//          from 2048 on, with 16 cells 1.07 to 1.6 up to 9216 and 0.90 to 0.95 from
+//          16384 on, with 8 cells 1.1 to 1.8; K = 4: 1.06 to 1.9 up to 4096, with up to
+//          16 cells 1.1 to 2.2
+//   p = 2, K = 1: 0.99 to 2.1 up to 2048 columns, 0.83 to 1.09 above; K = 2: 1.1 to 2.2
+//   p = 3, K = 1: 1.2 to 6 up to 102,400 cells or 16 subdomains, 0.55 to 0.91 above;
+//          K = 2: 1.2 to 8.6 up to 262,144 cells, 0.77 to 1.09 at 1024^2; K = 3: 0.99 to 10
 static bool split_pays(const kin_ctx* c)
 {
-    if (c->degree > 1 || std::min(c->L[0], c->L[1]) <= 16) return true;
-    return 3LL * c->m * c->tiles[0] * c->tiles[1] <= 152LL * std::max(1, 5 * c->iters - 9);
+    const int least = std::min(c->L[0], c->L[1]), K = c->iters;
+    const long long subs = (long long)c->tiles[0] * c->tiles[1], columns = subs * std::max(c->L[0], c->L[1]);
+    if (c->degree == 1) {
+        if (K == 1) return least > 8 && columns <= 256;
+        if (K == 2) return least <= 8 || columns <= 768;
+        if (K == 3) return least <= 8 || columns <= (least <= 16 ? 10000 : 2000);
+        return least <= 16 || columns <= 4096;
+    }
+    if (c->degree == 2) return K > 1 || columns <= 2048;
+    if (K == 1) return subs <= 16 || c->cells <= 110000;
+    return K > 2 || c->cells <= 400000;
 }
 
 // To be called before work that writes f is put on stream st.  Work captured
