@@ -118,7 +118,10 @@ typedef void (*kin_free_fn)(void* ptr, size_t bytes, void* stream, void* user);
  * subdomain extent n[a]/tiles[a]; 0 = chosen by the library).  The block
  * size changes only the schedule, never the result beyond round-off.
  * mem_budget: upper bound in bytes on device memory the context may hold
- * (0 = unbounded).  stream: cudaStream_t (NULL = the legacy default stream). */
+ * (0 = unbounded).  FP32 D2Q3 contexts keep records for a faster sweep, about as
+ * much again as f and W (kin_info.device_bytes), where that pays, the budget
+ * allows it and three quarters of the device's memory stay free; without them
+ * results agree to round-off.  stream: cudaStream_t (NULL = the legacy default stream). */
 typedef struct {
     int tiles[3];
     int iters;

@@ -73,7 +73,7 @@ struct kin_ctx {
     void* sxtr[2][3] = {};
     std::vector<double> sx_hrec;      // FP64 records [velocity][sx_stride], passed in the sweep parameters
     SxPlan sx_plan = {};
-    void* sxz = nullptr;              // split sweep (2D, FP32): records; NULL when they did not fit the budget
+    void* sxz = nullptr;              // split sweep (2D, FP32): records; NULL where it does not pay or memory is short
     int sxz_parity = 0;
     bool sxz_ready = false;           // the records are those of f
     bool sxz_captured = false;        // work that writes f was captured into a graph (note_capture)
@@ -950,9 +950,15 @@ static kin_status create_grid(const kin_mesh* mesh, const kin_model* model, int 
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess) {
             e = sx_sweep_plan(sx_args(c), c->precision == KIN_FP32, &c->sx_plan);
-            // (the records are an option: without room for them the one-kernel sweep runs)
+            // The records are an option (without room for them the one-kernel sweep
+            // runs), of about the size of everything else that the context holds.  So
+            // that they do not take the memory of contexts made later, they are only
+            // taken while three quarters of the device's memory stay free.
+            const size_t extra = sx_split_bytes(sx_args(c));
+            size_t mfree = 0, mtotal = 0;
+            if (e == cudaSuccess) e = cudaMemGetInfo(&mfree, &mtotal);
             if (e == cudaSuccess && c->dim == 2 && c->precision == KIN_FP32 && split_pays(c) &&
-                dev_alloc(c, sx_split_bytes(sx_args(c)), &c->sxz) == KIN_OK)
+                mfree > extra && mfree - extra >= mtotal / 4 * 3 && dev_alloc(c, extra, &c->sxz) == KIN_OK)
                 e = sx_split_plan(sx_args(c), &c->sx_plan);
             c->err.clear();
             c->grid = c->sx_plan.split ? c->sx_plan.bpv : c->nvel * c->sx_plan.bpv;
