@@ -964,6 +964,10 @@ static kin_status create_grid(const kin_mesh* mesh, const kin_model* model, int 
             c->grid = c->sx_plan.split ? c->sx_plan.bpv : c->nvel * c->sx_plan.bpv;
             c->threads = c->sx_plan.threads;
             c->smem = (int)c->sx_plan.smem;
+            if (c->sxz) {
+                c->grid = c->nvel * c->sx_plan.split_bpv;
+                c->smem = (int)c->sx_plan.split_smem;
+            }
         }
         if (e != cudaSuccess) {
             g_create_error = std::string("setup failed: ") + cudaGetErrorString(e);
@@ -1810,9 +1814,10 @@ kin_status kin_query(const kin_ctx* c, kin_info* info)
     info->device_bytes = c->bytes_held;
     info->precision = c->precision;
     for (int a = 0; a < 3; ++a) info->block[a] = c->B[a];
-    info->smem_bytes = c->smem;
-    info->grid = c->grid;
-    info->threads = c->threads;
+    // the launch that does a step's sweep
+    info->smem_bytes = c->multi ? (int)c->multi_smem : c->smem;
+    info->grid = c->multi ? c->multi_blocks : c->grid;
+    info->threads = c->multi ? kMultiThreads : c->threads;
     info->stages = c->stages;
     info->specialised = c->fixed ? 1 : 0;
     info->steps_done = c->steps_done;
