@@ -237,9 +237,13 @@ static bool choose_block(const kin_ctx* c, int B[3], bool thick)
         bool fits = true;
         for (int a = 0; a < 3; ++a)
             if (c->L[a] % shapes[k][a]) fits = false;
-        // FP64, 2D, p = 3: two waves of the fixed 8 x 4 tiles or the smaller tiles
-        // of the generic kernel -- 10 steps, 8 x 4 against 4 x 4: 16 to 64 tiles
-        // 461 and 308 us, 192 tiles 686 and 629, 384 tiles 1004 and 1112
+        // FP64, 2D, p = 3, fewer cells than two waves of 8 x 4 tiles: the small tiles
+        // that shrinking gives, whether 8 x 4 fits or not.  us per step, fixed 8 x 4
+        // against generic 4 x 4: up to 64 tiles 43 and 25, 128 43 and 37, 192 64 and 52,
+        // 288 66 and 66, 384 95 and 95, 2048 416 and 412.  On subdomains that 8 x 4 does
+        // not fit the estimate below is no better on the whole, shrunk against estimated: 50^2 cells
+        // in 25^2 28.9 and 35.1, 75^2 in 15^2 51.5 and 57.4, 69^2 in 23^2 72.7 and 71.9, 100^2
+        // in 25^2 92.4 and 79.6
         if (c->dim == 2 && c->esize == 8 && c->degree == 3 &&
             c->n[0] / shapes[k][0] * (c->n[1] / shapes[k][1]) < 2 * 152) {
             shrink_block(c, B);
@@ -355,7 +359,6 @@ static Inst make_inst(const kin_ctx* c, int mode)
     for (int a = 0; a < 3; ++a) I.fd_nb[a] = make_fastdiv((unsigned)c->nb[a]);
     I.fd_nrows = make_fastdiv((unsigned)(c->B[1] * c->B[2]));
     I.fd_B1 = make_fastdiv((unsigned)c->B[1]);
-    I.fd_rowlen = make_fastdiv((unsigned)(c->B[0] * c->NN));
     I.iters = c->iters;
     I.mode = mode;
     I.vec = rows_are_16b_aligned(c) ? 1 : 0;

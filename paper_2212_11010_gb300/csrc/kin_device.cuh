@@ -95,7 +95,6 @@ struct __align__(16) Inst {
     FastDiv fd_nb[3];        // nb[a]
     FastDiv fd_nrows;        // B[1] * B[2]
     FastDiv fd_B1;           // B[1]
-    FastDiv fd_rowlen;       // B[0] * nodes per cell
     int iters;               // K
     int mode;                // 0: full step, 1: summaries only (no transport, no store)
     int tma;                 // 1: rows moved by bulk copies (alignment checked on the host)
