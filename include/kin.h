@@ -145,7 +145,7 @@ typedef struct {
 enum { KIN_DEBUG_STALL_LOAD = 1 };
 
 /* Sizes of a context.  smem_bytes, grid and threads are those of the launch
- * that kin_step uses for its sweeps (1D: for all steps of a call). */
+ * that kin_step uses for its sweeps (1D: for the steps of a long call). */
 typedef struct {
     int dim, degree, m, nvel, npop, nodes_per_cell;
     size_t cells, nodes;            /* nodes = cells * nodes_per_cell          */

@@ -63,7 +63,7 @@ struct kin_ctx {
     bool fixed = false;                    // compile-time block shape kernel in use
     const void* multi = nullptr;           // several steps per launch (1D, kin_step_d1.cu)
     size_t multi_smem = 0;
-    int multi_blocks = 1;
+    int multi_blocks = 1, multi_from = 2;  // ... for calls of at least multi_from steps
     // d + 1 velocity sets
     bool simplex = false;
     int vsgn[4][3] = {};
@@ -487,6 +487,7 @@ static cudaError_t configure_launch(kin_ctx* c)
             c->multi = mk.fn;
             c->multi_smem = mk.smem;
             c->multi_blocks = mk.blocks;
+            c->multi_from = mk.from;
         }
     }
     return e;
@@ -1655,7 +1656,7 @@ kin_status kin_step(kin_ctx* c, int nsteps)
         if (st) return st;
         c->sum_stale = false;
     }
-    if (c->multi && nsteps > 0) {
+    if (c->multi && nsteps >= c->multi_from) {
         KIN_CUDA(c, launch_multi(c, make_inst(c, 0), nsteps, c->stream));
         c->cur ^= nsteps & 1;
         c->steps_done += nsteps;
@@ -1932,7 +1933,6 @@ static cudaError_t batch_launch(kin_batch* b, size_t k, int q, cudaStream_t st, 
         I.raw_out = c->raw[c->cur];
     }
     c->cur = saved;
-    if (c->multi && !prep) return launch_multi(c, I, 1, st);      // bitwise what kin_step does
     void* args[] = {&I};
     return cudaLaunchKernel((const void*)c->kfn, dim3(c->grid), dim3(c->threads), args, (size_t)c->smem, st);
 }

@@ -260,6 +260,7 @@ struct MultiKernel {
     const void* fn;
     size_t smem;
     int blocks;              // blocks of the cluster
+    int from;                // steps of a call from which it is used
 };
 MultiKernel multi_kernel_d1(int degree, int system, int prec, int n, int B);
 

@@ -197,7 +197,7 @@ static const void* multi_pick(int prec)
 
 MultiKernel multi_kernel_d1(int degree, int system, int prec, int n, int B)
 {
-    MultiKernel k{nullptr, 0, 1};
+    MultiKernel k{nullptr, 0, 1, 2};
     const int npop = 2 * nvars(1, system), np = degree + 1, nblk = n / B;
     const long long values = (long long)n * np * npop;
     if (values > (prec == 1 ? 65536 : 16384)) return k;
@@ -205,7 +205,17 @@ MultiKernel multi_kernel_d1(int degree, int system, int prec, int n, int B)
     // 10.3 to 12.2 us against 10.7 to 12.8 of one launch per step, and the gain
     // falls with the chain of a line)
     if (prec != 1 && B * np > 20) return k;
+    // (FP32, p = 1, 65536 values: 7.3 us per step either way)
+    if (prec == 1 && degree == 1 && values > 32768) return k;
     k.blocks = values <= (prec == 1 ? 3072 : 1536) ? 1 : 8;
+    // Calls of few steps take one launch of the grid-wide kernel per step (the results
+    // are bitwise the same): one block or cluster spends about 5 us on moving f in and
+    // out, the more the fewer values it shares the GPU for.  us of a call of n steps,
+    // here against there: FP32, 4096 to 24576 values 8 + 3 (n - 1) and 6.2 n; 32768 10 + 4
+    // (n - 1) and 6.2 n; 49152 12.3 + 6.0 (n - 1) and 6.2 n; FP64, 4096 to 8192 values 12
+    // to 16 + 8 to 10 (n - 1) and 10 to 12 n; 16384 16 to 18 + 9.9 to 11.8 (n - 1) and 10.3
+    // to 12.3 n.
+    if (k.blocks > 1) k.from = prec == 1 ? (values <= 24576 ? 2 : (values <= 32768 ? 4 : 33)) : (values <= 8192 ? 5 : 15);
     const int per = (nblk + k.blocks - 1) / k.blocks;
     k.smem = (size_t)(prec == 1 ? 4 : 8) * npop * ((size_t)4 * per + (size_t)per * B * np);
     if (k.smem > 200 * 1024 || npop * per > kMultiThreads) return k;
