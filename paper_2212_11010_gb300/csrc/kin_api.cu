@@ -322,6 +322,16 @@ static RelaxConsts relax_constants(const kin_ctx* c)
     return relax_consts(c->lambda, c->gamma, c->omega, mu, c->adv);
 }
 
+// Look-back depth of a direction: the fewest upstream blocks d with
+// |rho^B|^d <= tol, tol well below the rounding of the precision.
+static int lookback_depth(const kin_ctx* c, int d)
+{
+    const double tol = c->esize == 4 ? std::ldexp(1.0, -36) : std::ldexp(1.0, -72);
+    const double rb = std::fabs(c->coef_host[d][kOffRhoB]);
+    if (!(rb < 1.0)) return 1 << 30;                           // no truncation
+    return rb == 0.0 ? 1 : std::max(1, (int)std::ceil(std::log(tol) / std::log(rb)));
+}
+
 static Inst make_inst(const kin_ctx* c, int mode)
 {
     Inst I;
@@ -369,16 +379,25 @@ static Inst make_inst(const kin_ctx* c, int mode)
     I.rx = relax_constants(c);
     for (int a = 0; a < 3; ++a) I.inflow[a] = c->inflow[a];
     I.bnd = c->bnd_dev;
-    // look-back depth per direction: the fewest upstream blocks d with
-    // |rho^B|^d <= tol, tol well below the rounding of the precision
-    const double tol = c->esize == 4 ? std::ldexp(1.0, -36) : std::ldexp(1.0, -72);
-    for (int d = 0; d < 6; ++d) {
-        const double rb = std::fabs(c->coef_host[d][kOffRhoB]);
-        int depth = 1 << 30;                                   // no truncation
-        if (rb < 1.0) depth = rb == 0.0 ? 1 : std::max(1, (int)std::ceil(std::log(tol) / std::log(rb)));
-        I.lbdepth[d] = depth;
-    }
+    for (int d = 0; d < 6; ++d) I.lbdepth[d] = lookback_depth(c, d);
     return I;
+}
+
+// Whether a 1D call of nsteps steps takes one launch (c->multi).  Beside the number
+// of steps (MultiKernel::from) the length of the look-back decides: a block, or worse a
+// cluster, folds its summaries with few warps to hide one another's latency.  One
+// launch per step / one launch, 100 steps, subdomains of 17 to 358 cells in blocks of 1 to 3:
+// FP32 in one block 1.25 to 1.7 whatever the folds, in eight 1.12 to 2.1 up to 31 folds
+// and 0.81 to 1.13 at 60; FP64 in one block 1.16 to 1.38 up to 62 folds and 0.80 to 0.97
+// at 120, in eight 0.98 to 1.14 up to 41, 0.80 to 1.08 at 60, 0.71 to 0.89 at 120 -- but
+// 1.26 to 1.44 (FP32 1.43) where the grid-wide kernel takes two waves of tiles.
+static bool multi_pays(const kin_ctx* c, int nsteps)
+{
+    if (!c->multi || nsteps < c->multi_from) return false;
+    const long long whole = (2LL * c->iters - 1) * c->nb[0] / 2;       // (K - 1) nb + nb / 2 blocks
+    const long long folds = std::min<long long>(std::max(lookback_depth(c, 0), lookback_depth(c, 1)), whole);
+    if (c->multi_blocks == 1) return c->esize == 4 || folds <= 80;
+    return folds <= (c->esize == 4 ? 40 : 45) || c->nblk[0] > c->grid;
 }
 
 // Status of a device error word value h.
@@ -1656,7 +1675,7 @@ kin_status kin_step(kin_ctx* c, int nsteps)
         if (st) return st;
         c->sum_stale = false;
     }
-    if (c->multi && nsteps >= c->multi_from) {
+    if (multi_pays(c, nsteps)) {
         KIN_CUDA(c, launch_multi(c, make_inst(c, 0), nsteps, c->stream));
         c->cur ^= nsteps & 1;
         c->steps_done += nsteps;
@@ -1819,9 +1838,10 @@ kin_status kin_query(const kin_ctx* c, kin_info* info)
     info->precision = c->precision;
     for (int a = 0; a < 3; ++a) info->block[a] = c->B[a];
     // the launch that does a step's sweep
-    info->smem_bytes = c->multi ? (int)c->multi_smem : c->smem;
-    info->grid = c->multi ? c->multi_blocks : c->grid;
-    info->threads = c->multi ? kMultiThreads : c->threads;
+    const bool multi = multi_pays(c, INT_MAX);
+    info->smem_bytes = multi ? (int)c->multi_smem : c->smem;
+    info->grid = multi ? c->multi_blocks : c->grid;
+    info->threads = multi ? kMultiThreads : c->threads;
     info->stages = c->stages;
     info->specialised = c->fixed ? 1 : 0;
     info->steps_done = c->steps_done;

@@ -43,3 +43,14 @@ def test_chain_of_the_split_sweep(kin):
     # two parities of 8 + 4 record and 3 face values per lane, 32 cells' inflow and outflow faces
     assert split.smem_bytes == 4 * (2 * 32 * (12 + 3) + 2 * 32 * 3)
     assert split.smem_bytes != one.smem_bytes
+
+
+@pytest.mark.parametrize("prec,L,tiles,clustered", [("f64", 83, 4, False), ("f64", 64, 4, True), ("f64", 25, 4, True),
+                                                    ("f64", 67, 1, False), ("f32", 331, 4, False), ("f32", 83, 2, True),
+                                                    ("f64", 121, 8, True)])
+def test_long_lookbacks_take_one_launch_per_step(kin, prec, L, tiles, clustered):
+    # (blocks of one cell where the subdomain is a prime: 60 folds in FP32, 120 in FP64)
+    n = L * tiles
+    w = workloads.advection1d(seed=0, n=n, tiles=tiles, degree=3 if L == 121 else 1, dt=2.4 / n, precision=prec)
+    with kin.Context.from_workload(w) as ctx:
+        assert (ctx.info.threads == 512) == clustered
