@@ -387,6 +387,11 @@ struct SxWave {
     int bpv;            // thread blocks per velocity
     int k0;             // first velocity of this launch
     SxDiv div_nsub, div_ns0, div_ns1;
+    // The records are operands from the constant bank, and where they begin matters (56
+    // unused bytes, without -> with: 2D p = 3 FP32 310 -> 255 us per step of 512^2 cells
+    // (K = 1), 3D p = 2 FP32 3.25 -> 3.13 ms of 24^3, 3D p = 1 FP64 0.988 -> 0.966 of 32^3;
+    // but the bricks 26.91 -> 27.04 of 128^3, 12 steps).
+    int fill[D == 3 && P == 1 && sizeof(T) == 4 ? 0 : 14];
     T ainv[NV][NN * NN];
     T wcell[NN];
     T face[NV][D][TN];
