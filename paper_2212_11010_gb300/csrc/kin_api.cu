@@ -648,8 +648,11 @@ static SxArgs sx_args(const kin_ctx* c)
 //          16384 on, with 8 cells 1.1 to 1.8; K = 4: 1.06 to 1.9 up to 4096, with up to
 //          16 cells 1.1 to 2.2
 //   p = 2, K = 1: 0.99 to 2.1 up to 2048 columns, 0.83 to 1.09 above; K = 2: 1.1 to 2.2
-//   p = 3, K = 1: 1.2 to 6 up to 102,400 cells or 16 subdomains, 0.55 to 0.91 above;
-//          K = 2: 1.2 to 8.6 up to 262,144 cells, 0.77 to 1.09 at 1024^2; K = 3: 0.99 to 10
+//   p = 3, K = 1: with 8 cells 1.15 to 1.24; else 0.99 to 1.3 up to 36,864 cells and 0.52 to 0.88
+//          above, but 1.1 to 1.8 at 65,536 cells in at most 16 subdomains; K = 2: with up to 16
+//          cells 1.2 to 2.2; else 1.3 to 2.5 up to 102,400 cells, 0.73 to 1.1 above, but 1.2 up
+//          to 262,144 in at most 36 subdomains; K = 3: 1.07 to 3 up to 409,600 cells or with
+//          16 cells, 0.93 to 1.07 above; K = 4: 1.1 to 3.7
 static bool split_pays(const kin_ctx* c)
 {
     const int least = std::min(c->L[0], c->L[1]), K = c->iters;
@@ -661,8 +664,9 @@ static bool split_pays(const kin_ctx* c)
         return least <= 16 || columns <= 4096;
     }
     if (c->degree == 2) return K > 1 || columns <= 2048;
-    if (K == 1) return subs <= 16 || c->cells <= 110000;
-    return K > 2 || c->cells <= 400000;
+    if (K == 1) return least <= 8 || c->cells <= 40000 || (subs <= 16 && c->cells <= 70000);
+    if (K == 2) return least <= 16 || c->cells <= 110000 || (subs <= 40 && c->cells <= 270000);
+    return K > 3 || least <= 16 || c->cells <= 500000;
 }
 
 // To be called before work that writes f is put on stream st.  Work captured
