@@ -656,7 +656,8 @@ static SxArgs sx_args(const kin_ctx* c)
 static bool split_pays(const kin_ctx* c)
 {
     const int least = std::min(c->L[0], c->L[1]), K = c->iters;
-    const long long subs = (long long)c->tiles[0] * c->tiles[1], columns = subs * std::max(c->L[0], c->L[1]);
+    const long long subs = (long long)c->tiles[0] * c->tiles[1];
+    const double columns = subs * std::sqrt((double)c->L[0] * c->L[1]);      // of square subdomains of that size
     if (c->degree == 1) {
         if (K == 1) return least > 8 && columns <= 256;
         if (K == 2) return least <= 8 || columns <= 768;
