@@ -1631,7 +1631,10 @@ cudaError_t sx_sweep_plan(const SxArgs& a, int prec, SxPlan* plan)
     // columns, and enough of them that 16 warps per SM have work -- a brick wave
     // is eight cells long, and with few warps its latency shows (12 steps, one
     // cell against bricks: 22 warps per SM, 48^3 cells in 6^3 subdomains, 5.5 ms
-    // against 4.0; 7 per SM, 40 x 40 x 48 cells, 2.8 against 4.1).
+    // against 4.0; 7 per SM, 40 x 40 x 48 cells, 2.8 against 4.1).  True of up to 10
+    // columns; with 11 to 16 bricks are faster from about 96 warps per SM on and with 17 to 32
+    // from 108 (us per step, one cell against bricks: 8^3 cells, 343 subdomains 302 and 454,
+    // 729 707 and 717, 1331 1123 and 945; 12 x 10 x 8 cells, 180 307 and 533, 729 1157 and 1059).
     const bool even = a.dim == 3 && a.degree == 1 && a.L[0] % 2 == 0 && a.L[1] % 2 == 0 && a.L[2] % 2 == 0;
     const BrickShape bs = brick_shape(a.L[0], a.L[1]);
     const long long all = (long long)a.nvel * a.m * a.NS[0] * a.NS[1] * a.NS[2];
